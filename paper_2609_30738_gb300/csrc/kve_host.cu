@@ -40,14 +40,14 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-// [rows][128] bf16 viewed as a 2-D tensor; boxes of 64 elements x 128 rows with the
+// [rows][128] bf16 viewed as a 2-D tensor; boxes of 64 elements x box_rows rows with the
 // 128-byte swizzle, rows past the end read as zero.
-bool encode_rows(CUtensorMap* map, const void* base, int64_t rows) {
+bool encode_rows(CUtensorMap* map, const void* base, int64_t rows, int box_rows) {
   auto fn = encode_fn();
   if (!fn) return false;
   cuuint64_t dims[2] = {static_cast<cuuint64_t>(kHeadDim), static_cast<cuuint64_t>(rows)};
   cuuint64_t strides[1] = {static_cast<cuuint64_t>(kHeadDim) * 2};
-  cuuint32_t box[2] = {64, 128};
+  cuuint32_t box[2] = {64, static_cast<cuuint32_t>(box_rows)};
   cuuint32_t estr[2] = {1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -282,7 +282,7 @@ kve_status score_impl(const kve_plan* plan, const uint16_t* q_win, const uint16_
   if (sms <= 0) return KVE_ECUDA;
   CUtensorMap tm_q, tm_k, tm_v;
   const int64_t q_rows = static_cast<int64_t>(g.num_layers) * g.n_req * g.hq * g.window;
-  if (!encode_rows(&tm_q, q_win, q_rows) || !encode_keys(&tm_k, k, g)) return KVE_ECUDA;
+  if (!encode_rows(&tm_q, q_win, q_rows, kve::score_q_rows(g.n_rows, v != nullptr)) || !encode_keys(&tm_k, k, g)) return KVE_ECUDA;
   if (v && !encode_keys(&tm_v, v, g, true)) return KVE_ECUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   uint8_t* w = static_cast<uint8_t*>(ws);
@@ -303,7 +303,8 @@ kve_status score_impl(const kve_plan* plan, const uint16_t* q_win, const uint16_
   p.lse = lse;
   const int64_t ctas = std::min<int64_t>(sms, g.n_items);
   p.lag = score_lag(g, ctas);
-  if (kve::launch_score(*plan, tm_q, tm_k, v ? &tm_v : nullptr, p, static_cast<int>(ctas), st) != cudaSuccess)
+  p.heads = 1;
+  if (kve::launch_score(tm_q, tm_k, v ? &tm_v : nullptr, p, static_cast<int>(ctas), st) != cudaSuccess)
     return KVE_ECUDA;
   if (v && kve::launch_attn_finish(*plan, p.o_part, o_win, st) != cudaSuccess) return KVE_ECUDA;
   return KVE_OK;

@@ -124,6 +124,7 @@ struct ScoreParams {
   float alpha;               // log2(e) / sqrt(d)
   uint64_t wait_limit_ns;
   int32_t fault;             // test hook: 1 = unit 0 never publishes its statistics
+  int32_t heads;             // sets of rows with statistics of their own in a unit: 1, or 4 query heads
   int32_t lag;               // rounds a CTA's phase-1 item trails its phase-0 item
   float* mu;
   float* sigma;
@@ -228,8 +229,10 @@ cudaError_t launch_after_previous(void (*fn)(KArgs...), dim3 grid, dim3 block, s
 // Kernel launchers (defined next to their kernels).
 // tm_v = null: the plain score kernel; otherwise the variant that also accumulates the
 // window rows' attention output into p.o_part (then launch_attn_finish).
-cudaError_t launch_score(const kve_plan& plan, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
-                         const CUtensorMap* tm_v, const ScoreParams& p, int ctas, cudaStream_t stream);
+cudaError_t launch_score(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap* tm_v,
+                         const ScoreParams& p, int ctas, cudaStream_t stream);
+// Window rows that the score kernel loads for a unit of n_rows rows (the Q box of its TMA map).
+inline int score_q_rows(int n_rows, bool window_output) { return window_output || n_rows > 32 ? 128 : 32; }
 cudaError_t launch_attn_finish(const kve_plan& plan, const float* o_part, uint16_t* o_win,
                                cudaStream_t stream);
 cudaError_t launch_select(const kve_plan& plan, const SelectParams& p, cudaStream_t stream);

@@ -12,10 +12,11 @@
 //                               row; the item's (m, Z) per row are published, and
 //                               the last item of a unit to publish merges them into
 //                               beta_r = log2 of the row's softmax normaliser.
-//   phase 1 (column statistics): D[key][row] = K Q^T (keys on TMEM lanes); each
-//                               epilogue thread owns one key, forms
-//                               A = 2^(alpha*l - beta_r) for its n rows and reduces
-//                               them to mu and sigma in registers (sums and sums of
+//                               (Up to 32 rows both phases have the keys on the lanes.)
+//   phase 1 (column statistics): D[key][row] = K Q^T (keys on TMEM lanes); the
+//                               epilogue forms A = 2^(alpha*l - beta_r) for a key's n
+//                               rows, a quarter of them per thread (fragment loads),
+//                               and reduces them to mu and sigma (sums and sums of
 //                               squares; two passes where sigma/mu is small).
 // The schedule is static. CTA c owns items c, c + G, c + 2G, ... (G CTAs, all
 // resident: the launch is cooperative), so round j is items [jG, (j+1)G) and a
@@ -76,20 +77,34 @@ constexpr uint32_t kMNSbo = 1024;
 // buffer for 16 partials (measured: 1.84 ms per call at L = 32768 against 1.97 ms with
 // 2 Q buffers, 2 K stages and 8 partials); 3 score accumulators and the O^T accumulator
 // in TMEM columns 384..511.
-template <bool kAttn>
+// kRB: 32-row blocks that hold the unit's window rows, 1, 2 or 4. With one block the keys are the
+// M side of the MMA in both passes and N is 32; otherwise Q is loaded as 128 rows and the column
+// pass takes the first 32 kRB of them as N.
+template <int kRB, bool kAttn>
 struct Cfg {
+  static constexpr int kQRows = kRB == 1 ? 32 : 128;
+  static constexpr uint32_t kQHalf = kQRows * 128u;          // one 64-element column block of Q
+  static constexpr uint32_t kQBytes = 2 * kQHalf;
   static constexpr int kQBufs = kAttn ? 1 : 2;
-  static constexpr int kKStages = 3;
+  static constexpr int kKStages = kRB == 1 ? 4 : 3;
   static constexpr int kVStages = kAttn ? 2 : 0;
   static constexpr int kAccBufs = kAttn ? 3 : 4;
   static constexpr int kMergeBatch = kAttn ? 16 : 40;   // partials per bulk copy (1 KB each)
   static constexpr size_t kMergeBytes = static_cast<size_t>(kMergeBatch) * kMaxRows * sizeof(float2);
-  static constexpr size_t kDynSmem = (kQBufs + kKStages + kVStages) * kTileBytes + kMergeBytes + 1024;
+  static constexpr size_t kDynSmem =
+      kQBufs * kQBytes + (kKStages + kVStages) * kTileBytes + kMergeBytes + 1024;
+  // parts of a row item's (m, Z) that the epilogue leaves per row: one per epilogue group (a row
+  // per thread), or one per epilogue warp (keys on the lanes)
+  static constexpr int kParts = kRB == 1 ? kEpiWarps : 2;
+  static constexpr int kPartRows = kRB == 1 ? 32 : kMaxRows;
 };
-constexpr int kMaxKStages = 3;
-static_assert(Cfg<false>::kKStages <= kMaxKStages && Cfg<true>::kKStages <= kMaxKStages, "K stage arrays");
-static_assert(Cfg<true>::kVStages <= 2, "V stage arrays");
-static_assert(Cfg<false>::kQBufs <= kMaxQBufs && Cfg<true>::kQBufs <= kMaxQBufs, "Q buffer arrays");
+constexpr int kMaxKStages = 4;
+constexpr int kCombWords = 256;   // float2 of a row item: kParts * kPartRows
+static_assert(Cfg<1, false>::kParts * Cfg<1, false>::kPartRows == kCombWords &&
+              Cfg<4, false>::kParts * Cfg<4, false>::kPartRows == kCombWords, "comb");
+static_assert(Cfg<1, false>::kKStages <= kMaxKStages && Cfg<4, true>::kKStages <= kMaxKStages, "K stage arrays");
+static_assert(Cfg<4, true>::kVStages <= 2, "V stage arrays");
+static_assert(Cfg<4, false>::kQBufs <= kMaxQBufs && Cfg<4, true>::kQBufs <= kMaxQBufs, "Q buffer arrays");
 constexpr int kMaxAccBufs = 4;
 constexpr uint32_t kOCol = 384;   // TMEM column of the O^T accumulator (window output)
 
@@ -140,8 +155,7 @@ struct ScoreCtl {
   uint32_t tmem_base;
   volatile int abort;
   int32_t roww[kMaxRows];                            // r % W
-  float rowm[kMaxRows];                              // 1 for rows r < n, else 0
-  alignas(16) float2 comb[kItemSlots][2][kMaxRows];  // per group (m, Z) of a row item
+  alignas(16) float2 comb[kItemSlots][kCombWords];   // (m, Z) parts of a row item, [part][row]
   alignas(16) float nbeta[kItemSlots][kMaxRows];     // kColScale - beta of a column item
 };
 static_assert(offsetof(ScoreCtl, nbeta) % 16 == 0, "nbeta is read with 16-byte loads");
@@ -173,10 +187,11 @@ __device__ __forceinline__ float2 merge_mz(float2 a, float2 b) {
 
 // ---------------------------------------------------------------- epilogue, phase 0
 
-template <bool kFull, bool kAttn>
-__device__ __forceinline__ bool rowstats_item(const ScoreParams& P, ScoreCtl& ctl,
-                                              const ItemDesc& d, uint32_t slot, uint32_t& ai) {
-  constexpr int kAccBufs = Cfg<kAttn>::kAccBufs;
+// Rows on the lanes (more than 32 rows): the thread owns one row.
+template <bool kAttn>
+__device__ __forceinline__ bool rowstats_by_row(const ScoreParams& P, ScoreCtl& ctl,
+                                                const ItemDesc& d, uint32_t slot, uint32_t& ai) {
+  constexpr int kAccBufs = Cfg<4, kAttn>::kAccBufs;
   const int quad = (threadIdx.x >> 5) & 3;
   const int lane = threadIdx.x & 31;
   const int grp = (threadIdx.x - kEpiWarp0 * 32) >> 7;   // 0 or 1
@@ -239,7 +254,84 @@ __device__ __forceinline__ bool rowstats_item(const ScoreParams& P, ScoreCtl& ct
       m = mn;
     }
   }
-  ctl.comb[slot][grp][row] = make_float2(m, Z);
+  ctl.comb[slot][grp * kMaxRows + row] = make_float2(m, Z);
+  return true;
+}
+
+// One step of a reduction over lanes that also halves the values held: of (a, b) the lane
+// keeps one, by `hi`, and merges its partner's copy of it.
+__device__ __forceinline__ float2 merge_halves(float2 a, float2 b, bool hi, int mask) {
+  const float2 keep = hi ? b : a, give = hi ? a : b;
+  const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, give.x, mask),
+                                 __shfl_xor_sync(0xffffffffu, give.y, mask));
+  return merge_mz(keep, got);
+}
+
+// Keys on the lanes (at most 32 rows: with rows on the lanes three quarters of them or more
+// would compute rows that are not there). The fragment loads give thread (g, t) the keys g,
+// g + 8, g + 16, g + 24 of its warp's 32 and the rows 8c + 2t, 8c + 2t + 1; it keeps (m, Z) of
+// those 8 rows over its keys, and the warp merges them at the end of the item. Both passes of a
+// tile then cost a quarter of the exponentials, and a quarter of the MMA's N: 32 layers of 15611
+// tokens with 8 x 4 rows take 248 us of score kernel against 289.
+__device__ __forceinline__ bool rowstats_by_key(const ScoreParams& P, ScoreCtl& ctl,
+                                                const ItemDesc& d, uint32_t slot, uint32_t& ai) {
+  constexpr int kAccBufs = Cfg<1, false>::kAccBufs;
+  constexpr int kCols = 8;   // rows per thread
+  const int quad = (threadIdx.x >> 5) & 3;
+  const int lane = threadIdx.x & 31;
+  const int grp = (threadIdx.x - kEpiWarp0 * 32) >> 7;
+  const int g = lane >> 2, tq = lane & 3;
+  const int lim_all = d.L - P.g.window;
+  const int tile0 = d.tile0, ntiles = d.ntiles;
+  const float alpha = P.alpha;
+  const uint32_t tl = ctl.tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
+  float2 mz[kCols];
+#pragma unroll
+  for (int j = 0; j < kCols; ++j) mz[j] = make_float2(-INFINITY, 0.f);
+  for (int t = 0; t < ntiles; ++t, ++ai) {
+    if (static_cast<int>(ai & 1u) != grp) continue;
+    const uint32_t ab = ai % kAccBufs;
+    if (!warp_wait(&ctl.acc_full[ab], (ai / kAccBufs) & 1u, P.wait_limit_ns, &ctl.abort)) return false;
+    tc_fence_after();
+    float v[2][16];
+    tmem_ld16_x4(tl + ab * 128u, v[0]);
+    tmem_ld16_x4(tl + (16u << 16) + ab * 128u, v[1]);
+    tmem_wait_ld(v[0]);
+    tmem_wait_ld(v[1]);
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&ctl.acc_empty[ab]);
+    const int key0 = (tile0 + t) * kTileKeys;
+    if (__builtin_expect(key0 + kTileKeys - 1 > lim_all, 0)) {
+      const int key = key0 + quad * 32 + g;   // and + 8, + 16, + 24
+#pragma unroll
+      for (int j = 0; j < kCols; ++j) {
+        const int lim = lim_all + ctl.roww[8 * (j >> 1) + 2 * tq + (j & 1)];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (key + 8 * q > lim) v[q >> 1][4 * (j >> 1) + 2 * (q & 1) + (j & 1)] = -INFINITY;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kCols; ++j) {
+      const int c = 4 * (j >> 1) + (j & 1);
+      const float x0 = v[0][c], x1 = v[0][c + 2], x2 = v[1][c], x3 = v[1][c + 2];
+      const float mn = fmaxf(mz[j].x, max3(fmaxf(x0, x1), x2, x3) * alpha);
+      const float ref = mn == -INFINITY ? 0.f : mn;   // no key seen yet: every term below is 0
+      const float e01 = ex2(fmaf(x0, alpha, -ref)) + ex2(fmaf(x1, alpha, -ref));
+      const float e23 = ex2(fmaf(x2, alpha, -ref)) + ex2(fmaf(x3, alpha, -ref));
+      mz[j].y = fmaf(mz[j].y, ex2(mz[j].x - ref), e01 + e23);
+      mz[j].x = mn;
+    }
+  }
+  // over the 8 lanes of a row set: lane (g, t) ends with row 8 (g / 2) + 2 t + g % 2
+  float2 r4[4], r2[2];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) r4[j] = merge_halves(mz[j], mz[j + 4], (g & 4) != 0, 16);
+#pragma unroll
+  for (int j = 0; j < 2; ++j) r2[j] = merge_halves(r4[j], r4[j + 2], (g & 2) != 0, 8);
+  ctl.comb[slot][(grp * 4 + quad) * 32 + 8 * (g >> 1) + 2 * tq + (g & 1)] =
+      merge_halves(r2[0], r2[1], (g & 1) != 0, 4);
   return true;
 }
 
@@ -320,15 +412,15 @@ __device__ __forceinline__ void write_pt_half(uint8_t* pt, int key, int h0, cons
 }
 
 // Sum and sum of squares of a half (3 fp32 operations per element with the
-// exponent's argument: the FMA pipe stays below the MUFU pipe). With the window
-// output (pt != null), the half's probabilities also go to the P^T tile.
-template <bool kFull, bool kAttn>
+// exponent's argument: the FMA pipe stays below the MUFU pipe); the half's probabilities
+// also go to the P^T tile.
+template <bool kFull>
 __device__ __forceinline__ void colsums_half(const ScoreParams& P, const ScoreCtl& ctl,
                                              const float4* nb4, uint32_t taddr, int h0, int n,
                                              int rel, float& sum, float& sumsq, uint8_t* pt, int key) {
   float v[64];
   col_half_values<kFull>(P, ctl, nb4, taddr, h0, n, rel, v);
-  if constexpr (kAttn) write_pt_half(pt, key, h0, v);
+  write_pt_half(pt, key, h0, v);
   float2 c0 = make_float2(0.f, 0.f), c1 = c0, c2 = c0, c3 = c0;
   float2 q0 = c0, q1 = c0, q2 = c0, q3 = c0;
 #pragma unroll
@@ -350,47 +442,233 @@ __device__ __forceinline__ void colsums_half(const ScoreParams& P, const ScoreCt
   sumsq = qs.x + qs.y;
 }
 
-// The same half, two passes: its sum and its sum of squared deviations from its own
-// mean (no cancellation; used when the one-pass form cannot be trusted).
-template <bool kFull>
-__device__ __forceinline__ void colstats_half(const ScoreParams& P, const ScoreCtl& ctl,
-                                              const float4* nb4, uint32_t taddr, int h0, int n,
-                                              int rel, float& sum, float& m2) {
-  const int nh = kFull ? 64 : (n - h0 < 64 ? n - h0 : 64);
-  float v[64];
-  col_half_values<kFull>(P, ctl, nb4, taddr, h0, n, rel, v);
-  float2 c0 = make_float2(0.f, 0.f), c1 = c0, c2 = c0, c3 = c0;
-#pragma unroll
-  for (int r = 0; r < 64; r += 8) {
-    c0 = fadd2(c0, make_float2(v[r], v[r + 1]));
-    c1 = fadd2(c1, make_float2(v[r + 2], v[r + 3]));
-    c2 = fadd2(c2, make_float2(v[r + 4], v[r + 5]));
-    c3 = fadd2(c3, make_float2(v[r + 6], v[r + 7]));
+// Sum and sum of squared deviations of rows r0 .. r0 + rows - 1 of the lane's key, two passes
+// over chunks of at most 32 rows (no cancellation), the chunks combined by the pairwise update
+// of the mean and the sum of squared deviations (Chan, Golub, LeVeque). Used where the
+// one-pass form cannot be trusted, and for the tiles that hold window keys (their causal mask).
+__device__ __forceinline__ float2 colstats_exact(const ScoreParams& P, const ScoreCtl& ctl, const float4* nb4,
+                                                 uint32_t taddr, int r0, int rows, int rel) {
+  float S = 0.f, M2 = 0.f, cnt = 0.f;
+  // rows that see the key: those with row % W >= rel; where W divides 32 the same bits in every
+  // chunk (r0 is a multiple of W), otherwise looked up below
+  const int W = P.g.window;
+  const bool periodic = W <= 32 && (W & (W - 1)) == 0;
+  uint32_t sees = 0xFFFFFFFFu;
+  if (rel > 0 && periodic) {
+    sees = rel >= W ? 0u : (0xFFFFFFFFu >> (32 - W)) & (0xFFFFFFFFu << rel);
+    for (int w = W; w < 32; w <<= 1) sees |= sees << w;
   }
-  const float2 cs = fadd2(fadd2(c0, c1), fadd2(c2, c3));
-  sum = cs.x + cs.y;
-  const float mh = sum / static_cast<float>(nh);
-  float q = 0.f;
+#pragma unroll 1
+  for (int i = 0; i < rows; i += 32) {
+    const int nh = rows - i < 32 ? rows - i : 32;
+    float v[32];
+    tmem_ld32(taddr + static_cast<uint32_t>(r0 + i), v);
+    tmem_wait_ld(v);
+    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
 #pragma unroll
-  for (int r = 0; r < 64; ++r) {
-    // rows past n: no term (ctl.rowm is 1 for rows r < n, else 0)
-    const float d = kFull ? v[r] - mh : (v[r] - mh) * ctl.rowm[h0 + r];
-    q = fmaf(d, d, q);
+    for (int r = 0; r < 32; r += 4) {
+      const float4 b = nb4[(r0 + i + r) >> 2];
+      // columns past the rows may hold anything: no term, whatever their value
+      v[r] = r < nh && ((sees >> (r)) & 1u) ? ex2(fmaxf(fmaf(v[r], P.alpha, b.x), -INFINITY)) : 0.f;
+      v[r + 1] = r + 1 < nh && ((sees >> (r + 1)) & 1u) ? ex2(fmaxf(fmaf(v[r + 1], P.alpha, b.y), -INFINITY)) : 0.f;
+      v[r + 2] = r + 2 < nh && ((sees >> (r + 2)) & 1u) ? ex2(fmaxf(fmaf(v[r + 2], P.alpha, b.z), -INFINITY)) : 0.f;
+      v[r + 3] = r + 3 < nh && ((sees >> (r + 3)) & 1u) ? ex2(fmaxf(fmaf(v[r + 3], P.alpha, b.w), -INFINITY)) : 0.f;
+    }
+    if (!periodic && rel > 0) {
+#pragma unroll
+      for (int r = 0; r < 32; ++r)
+        if (r < nh && rel > ctl.roww[r0 + i + r]) v[r] = 0.f;   // the row does not see the key
+    }
+#pragma unroll
+    for (int r = 0; r < 32; r += 4) {
+      s0 += v[r];
+      s1 += v[r + 1];
+      s2 += v[r + 2];
+      s3 += v[r + 3];
+    }
+    const float fh = static_cast<float>(nh), sum = (s0 + s1) + (s2 + s3), mean = sum / fh;
+    float q = 0.f;
+#pragma unroll
+    for (int r = 0; r < 32; ++r) {
+      const float dv = r < nh ? v[r] - mean : 0.f;
+      q = fmaf(dv, dv, q);
+    }
+    if (i > 0) {
+      const float dd = mean - S / cnt;
+      q = fmaf(dd * dd, cnt * fh / (cnt + fh), q);
+    }
+    S += sum;
+    M2 += q;
+    cnt += fh;
   }
-  m2 = q;
+  return make_float2(S, M2);
 }
 
-// With the window output (kAttn), every tile's probabilities go to the P^T tile in the
+// Column statistics of an item by fragment loads: thread (g, t) gets the keys g and g + 8 of 16
+// keys at a time, and the rows 8c + 2t, 8c + 2t + 1 of every 8-row block c. It needs the
+// normalisers of those 8 kRB rows alone, which stay in registers for the whole item: with a key
+// per thread the epilogue reads every row's from shared memory for every tile, in competition
+// with the tensor cores' operand reads (128 bytes a cycle, which keep that port full while an
+// MMA runs). The loop over the two key halves is rolled: the row and column bodies alternate
+// item by item, and the unrolled form lost more in instruction fetch than it gained (642 against
+// 580 us). Against a key per thread, at 32 layers of 32768 tokens: two passes 580 us against 601,
+// given normalisers 337 against 343. The four lanes of a key are reduced after each half; lane
+// (g, t) keeps key g + 8 (t / 2) + 16 (t % 2). kHeads = 4: the rows are those of four query heads
+// that each have statistics of their own (equal runs of whole 8-row blocks).
+template <int kRB, bool kFull, int kHeads>
+__device__ __forceinline__ bool colstats_by_fragment(const ScoreParams& P, ScoreCtl& ctl,
+                                                     const ItemDesc& d, uint32_t slot, uint32_t& ai) {
+  constexpr int kAccBufs = Cfg<kRB, false>::kAccBufs;
+  constexpr int kBlocks = kRB == 1 ? 4 : 8;          // 8-row blocks per load
+  constexpr int kLoads = kRB == 4 ? 2 : 1;           // loads per 16 keys
+  constexpr int kBH = kHeads == 1 ? kBlocks : kRB;   // blocks of one head in a load
+  constexpr int kHL = kBlocks / kBH;                 // heads per load
+  const int quad = (threadIdx.x >> 5) & 3;
+  const int lane = threadIdx.x & 31;
+  const int grp = (threadIdx.x - kEpiWarp0 * 32) >> 7;
+  const int tq = lane & 3;
+  const int n = (kFull ? 32 * kRB : P.g.n_rows) / kHeads;   // rows of one set of statistics
+  const float fn = static_cast<float>(n);
+  const float inv_n = 1.0f / fn;
+  const float inv_n1 = n > 1 ? 1.0f / static_cast<float>(n - 1) : 0.f;
+  const int tile0 = d.tile0, ntiles = d.ntiles;
+  const int lim_all = d.L - P.g.window;
+  const float2 a2 = make_float2(P.alpha, P.alpha);
+  const float4* nb4 = reinterpret_cast<const float4*>(ctl.nbeta[slot]);
+  float2 nb[4 * kRB];
+#pragma unroll
+  for (int c = 0; c < 4 * kRB; ++c) nb[c] = *reinterpret_cast<const float2*>(&ctl.nbeta[slot][8 * c + 2 * tq]);
+  const uint32_t tl = ctl.tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
+  // the lane that keeps key `lane` of the quadrant's 32
+  const int owner = 4 * (lane & 7) + 2 * ((lane >> 3) & 1) + (lane >> 4);
+  for (int t = 0; t < ntiles; ++t, ++ai) {
+    if (static_cast<int>(ai & 1u) != grp) continue;
+    const uint32_t ab = ai % kAccBufs;
+    if (!warp_wait(&ctl.acc_full[ab], (ai / kAccBufs) & 1u, P.wait_limit_ns, &ctl.abort)) return false;
+    tc_fence_after();
+    const int key0 = (tile0 + t) * kTileKeys + quad * 32;
+    // a tile that holds window keys, which not every row sees, takes the exact form
+    const bool masked = (tile0 + t + 1) * kTileKeys - 1 > lim_all;
+    float S1[kHeads], m2[kHeads];
+    uint32_t exact = masked ? (1u << kHeads) - 1u : 0u;   // sets of this lane's key that need it
+#pragma unroll
+    for (int h = 0; h < kHeads; ++h) S1[h] = m2[h] = 0.f;
+    if (__builtin_expect(!masked, 1)) {
+#pragma unroll 1
+      for (int hh = 0; hh < 2; ++hh) {
+        float S[kHeads][2], Q[kHeads][2];   // keys g and g + 8
+#pragma unroll
+        for (int i = 0; i < kLoads; ++i) {
+          float v[4 * kBlocks];
+          const uint32_t ta = tl + (static_cast<uint32_t>(16 * hh) << 16) + ab * 128u + 64u * i;
+          if constexpr (kBlocks == 4) tmem_ld16_x4(ta, v); else tmem_ld16_x8(ta, v);
+          tmem_wait_ld(v);
+#pragma unroll
+          for (int hl = 0; hl < kHL; ++hl) {
+            float2 c0 = make_float2(0.f, 0.f), c1 = c0, c2 = c0, c3 = c0;
+            float2 q0 = c0, q1 = c0, q2 = c0, q3 = c0;
+#pragma unroll
+            for (int b = hl * kBH; b < (hl + 1) * kBH; ++b) {
+              const float2 nn = nb[8 * i + b];
+              float2 x0 = ffma2(make_float2(v[4 * b], v[4 * b + 1]), a2, nn);
+              float2 x1 = ffma2(make_float2(v[4 * b + 2], v[4 * b + 3]), a2, nn);
+              if constexpr (!kFull) {
+                // rows past n are staged as -inf: 2^-inf = 0 even where their products are not finite
+                x0 = make_float2(fmaxf(x0.x, -INFINITY), fmaxf(x0.y, -INFINITY));
+                x1 = make_float2(fmaxf(x1.x, -INFINITY), fmaxf(x1.y, -INFINITY));
+              }
+              x0 = make_float2(ex2(x0.x), ex2(x0.y));
+              x1 = make_float2(ex2(x1.x), ex2(x1.y));
+              if (kBH > 1 && (b & 1) != 0) {
+                c2 = fadd2(c2, x0);
+                c3 = fadd2(c3, x1);
+                q2 = ffma2(x0, x0, q2);
+                q3 = ffma2(x1, x1, q3);
+              } else {
+                c0 = fadd2(c0, x0);
+                c1 = fadd2(c1, x1);
+                q0 = ffma2(x0, x0, q0);
+                q1 = ffma2(x1, x1, q1);
+              }
+            }
+            if constexpr (kBH > 1) {
+              c0 = fadd2(c0, c2);
+              c1 = fadd2(c1, c3);
+              q0 = fadd2(q0, q2);
+              q1 = fadd2(q1, q3);
+            }
+            const int h = kHeads == 1 ? 0 : i * kHL + hl;
+            const bool more = kHeads == 1 && i > 0;
+            S[h][0] = more ? S[h][0] + (c0.x + c0.y) : c0.x + c0.y;
+            S[h][1] = more ? S[h][1] + (c1.x + c1.y) : c1.x + c1.y;
+            Q[h][0] = more ? Q[h][0] + (q0.x + q0.y) : q0.x + q0.y;
+            Q[h][1] = more ? Q[h][1] + (q1.x + q1.y) : q1.x + q1.y;
+          }
+        }
+        const bool hi = (tq & 2) != 0;
+#pragma unroll
+        for (int h = 0; h < kHeads; ++h) {
+          float a = (hi ? S[h][1] : S[h][0]) + __shfl_xor_sync(0xffffffffu, hi ? S[h][0] : S[h][1], 2);
+          float q = (hi ? Q[h][1] : Q[h][0]) + __shfl_xor_sync(0xffffffffu, hi ? Q[h][0] : Q[h][1], 2);
+          a += __shfl_xor_sync(0xffffffffu, a, 1);
+          q += __shfl_xor_sync(0xffffffffu, q, 1);
+          if ((tq & 1) == hh) {
+            S1[h] = a;
+            m2[h] = q;
+          }
+        }
+      }
+      // The one-pass form loses about (sum A'^2) * 2^-19 to rounding. It is kept while
+      // sigma^2 >= kOnePassMin * mu^2, where that loss stays below 2e-4 of sigma^2; otherwise
+      // (columns of nearly equal A, e.g. uniform attention) the warp takes the two-pass form
+      // over the same TMEM columns.
+#pragma unroll
+      for (int h = 0; h < kHeads; ++h) {
+        S1[h] = __shfl_sync(0xffffffffu, S1[h], owner);   // from here on a lane's key is its own
+        m2[h] = __shfl_sync(0xffffffffu, m2[h], owner);
+        m2[h] = fmaf(-S1[h], S1[h] * inv_n, m2[h]);
+        if (!(m2[h] * fn * fn >= kOnePassMin * (fn - 1.f) * S1[h] * S1[h])) exact |= 1u << h;   // NaN-safe
+      }
+    }
+    if (__builtin_expect(__any_sync(0xffffffffu, exact != 0u), 0)) {
+#pragma unroll 1
+      for (int h = 0; h < kHeads; ++h) {
+        const float2 e = colstats_exact(P, ctl, nb4, tl + ab * 128u, h * n, n, key0 + lane - lim_all);
+#pragma unroll
+        for (int j = 0; j < kHeads; ++j)
+          if (j == h && ((exact >> j) & 1u) != 0u) {
+            if (masked) S1[j] = e.x;
+            m2[j] = e.y;
+          }
+      }
+    }
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&ctl.acc_empty[ab]);
+    const int key = key0 + lane;
+    if (key < d.L) {
+#pragma unroll
+      for (int h = 0; h < kHeads; ++h) {
+        const int64_t at = d.mu_off + static_cast<int64_t>(h) * d.L + key;
+        __stcs(&P.mu[at], S1[h] * inv_n * kColUnscale);
+        __stcs(&P.sigma[at], sqrtf(fmaxf(m2[h], 0.f) * inv_n1) * kColUnscale);
+      }
+    }
+  }
+  return true;
+}
+
+// With the window output, a key per thread: every tile's probabilities go to the P^T tile in the
 // tile's K stage (kbuf + stage * 32 KB; the score MMA has finished with its K), announced
 // on p_full[stage]; at the end of the item group 0 reads the item's O^T accumulator
 // (lane = d, column = row) into o_part[item][row][d] and hands it back on o_empty. oi
 // counts the column items before this one.
-template <bool kFull, bool kAttn>
-__device__ __forceinline__ bool colstats_item(const ScoreParams& P, ScoreCtl& ctl,
+template <bool kFull>
+__device__ __forceinline__ bool colstats_with_output(const ScoreParams& P, ScoreCtl& ctl,
                                               const ItemDesc& d, uint32_t slot, uint32_t& ai,
                                               uint8_t* kbuf, uint32_t& oi) {
-  constexpr int kAccBufs = Cfg<kAttn>::kAccBufs;
-  constexpr int kKStages = Cfg<kAttn>::kKStages;
+  constexpr int kAccBufs = Cfg<4, true>::kAccBufs;
+  constexpr int kKStages = Cfg<4, true>::kKStages;
   const int quad = (threadIdx.x >> 5) & 3;
   const int lane = threadIdx.x & 31;
   const int grp = (threadIdx.x - kEpiWarp0 * 32) >> 7;
@@ -415,27 +693,25 @@ __device__ __forceinline__ bool colstats_item(const ScoreParams& P, ScoreCtl& ct
     // of squares, m2 = sum A'^2 - (sum A')^2 / n
     const bool two = kFull || n > 64;
     float S1 = 0.f, SS = 0.f;
-    uint8_t* pt = kAttn ? kbuf + (ai % kKStages) * kTileBytes : nullptr;
+    uint8_t* pt = kbuf + (ai % kKStages) * kTileBytes;
 #pragma unroll 1
     for (int h = 0; h < (two ? 2 : 1); ++h) {
       float sh, qh;
-      colsums_half<kFull, kAttn>(P, ctl, nb4, taddr, 64 * h, n, rel, sh, qh, pt, tl);
+      colsums_half<kFull>(P, ctl, nb4, taddr, 64 * h, n, rel, sh, qh, pt, tl);
       S1 += sh;
       SS += qh;
     }
-    if constexpr (kAttn) {
-      if (!two) {
-        // rows 64..127 are past n: their probabilities are 0
+    if (!two) {
+      // rows 64..127 are past n: their probabilities are 0
 #pragma unroll
-        for (int c = 0; c < 8; ++c)
-          *reinterpret_cast<uint4*>(pt + kHalfBytes + (tl >> 3) * 1024 + (tl & 7) * 128 + (c << 4)) =
-              make_uint4(0, 0, 0, 0);
-      }
-      // P^T is read by the tensor cores (async proxy) once every warp has announced it
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&ctl.p_full[ai % kKStages]);
+      for (int c = 0; c < 8; ++c)
+        *reinterpret_cast<uint4*>(pt + kHalfBytes + (tl >> 3) * 1024 + (tl & 7) * 128 + (c << 4)) =
+            make_uint4(0, 0, 0, 0);
     }
+    // P^T is read by the tensor cores (async proxy) once every warp has announced it
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&ctl.p_full[ai % kKStages]);
     float m2 = fmaf(-S1, S1 * inv_n, SS);
     // The one-pass form loses about (sum A'^2) * 2^-19 to rounding. It is kept while
     // sigma^2 >= kOnePassMin * mu^2, where that loss stays below 2e-4 of sigma^2;
@@ -444,20 +720,7 @@ __device__ __forceinline__ bool colstats_item(const ScoreParams& P, ScoreCtl& ct
     // update of the mean and the sum of squared deviations (Chan, Golub, LeVeque).
     const bool exact = !(m2 * fn * fn >= kOnePassMin * (fn - 1.f) * S1 * S1);   // NaN-safe
     if (__any_sync(0xffffffffu, exact)) {
-      float hs[2] = {0.f, 0.f}, hm2[2] = {0.f, 0.f};
-#pragma unroll 1
-      for (int h = 0; h < (two ? 2 : 1); ++h) {
-        float sh, mh2;
-        colstats_half<kFull>(P, ctl, nb4, taddr, 64 * h, n, rel, sh, mh2);
-        if (h == 0) { hs[0] = sh; hm2[0] = mh2; } else { hs[1] = sh; hm2[1] = mh2; }
-      }
-      const float n1 = kFull ? 64.f : static_cast<float>(n < 64 ? n : 64);
-      const float n2 = fn - n1;
-      float m2x = hm2[0] + hm2[1];
-      if (two) {
-        const float dd = hs[1] / n2 - hs[0] / n1;
-        m2x = fmaf(dd * dd, n1 * n2 * inv_n, m2x);
-      }
+      const float m2x = colstats_exact(P, ctl, nb4, taddr, 0, n, rel).y;
       if (exact) m2 = m2x;
     }
     tc_fence_before();
@@ -470,27 +733,25 @@ __device__ __forceinline__ bool colstats_item(const ScoreParams& P, ScoreCtl& ct
       __stcs(&P.sigma[d.mu_off + key], sigma);
     }
   }
-  if constexpr (kAttn) {
-    if (grp == 0) {
-      // the item's O^T (lane = d, column = row) into o_part[item][row][d]
-      if (!warp_wait(&ctl.o_full, oi & 1u, P.wait_limit_ns, &ctl.abort)) return false;
-      tc_fence_after();
-      const uint32_t taddr = ctl.tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + kOCol;
-      float* dst = P.o_part + d.p * (kMaxRows * kHeadDim) + tl;
+  if (grp == 0) {
+    // the item's O^T (lane = d, column = row) into o_part[item][row][d]
+    if (!warp_wait(&ctl.o_full, oi & 1u, P.wait_limit_ns, &ctl.abort)) return false;
+    tc_fence_after();
+    const uint32_t taddr = ctl.tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + kOCol;
+    float* dst = P.o_part + d.p * (kMaxRows * kHeadDim) + tl;
 #pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
-        float v[32];
-        tmem_ld32(taddr + 32u * c, v);
-        tmem_wait_ld();
+    for (int c = 0; c < 4; ++c) {
+      float v[32];
+      tmem_ld32(taddr + 32u * c, v);
+      tmem_wait_ld(v);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) __stcg(dst + (32 * c + j) * kHeadDim, v[j]);
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&ctl.o_empty);
+      for (int j = 0; j < 32; ++j) __stcg(dst + (32 * c + j) * kHeadDim, v[j]);
     }
-    ++oi;
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&ctl.o_empty);
   }
+  ++oi;
   return true;
 }
 
@@ -524,21 +785,30 @@ __device__ __forceinline__ bool stage_beta(const ScoreParams& P, ScoreCtl& ctl,
   return true;
 }
 
-// Phase-0 item: merge the two groups' (m, Z) per row, publish them and count the
+// Phase-0 item: merge the epilogue's parts of (m, Z) per row, publish them and count the
 // item. Returns whether it was the unit's last item to arrive. When the next ring
 // item is a phase-1 item not yet staged (next_unit >= 0), its normalisers are loaded
 // before the publication's fence and checked after its atomic (the round trips
 // overlap); *next_staged tells whether they were ready and are now staged.
+template <class C>
 __device__ __forceinline__ bool sync_rowstats(const ScoreParams& P, ScoreCtl& ctl,
                                               const ItemDesc& d, uint32_t slot, int64_t next_unit,
                                               uint32_t next_slot, bool* next_staged) {
   const int lane = threadIdx.x & 31;
   const int n = P.g.n_rows;
-  float2 mz[4];
+  constexpr int kRowSets = C::kPartRows / 32;
+  float2 mz[kRowSets];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int row = lane + 32 * k;
-    mz[k] = merge_mz(ctl.comb[slot][0][row], ctl.comb[slot][1][row]);
+  for (int k = 0; k < kRowSets; ++k) {
+    const float2* part = &ctl.comb[slot][lane + 32 * k];
+    float2 x[C::kParts];
+#pragma unroll
+    for (int j = 0; j < C::kParts; ++j) x[j] = part[j * C::kPartRows];
+#pragma unroll
+    for (int w = C::kParts / 2; w >= 1; w /= 2)
+#pragma unroll
+      for (int j = 0; j < w; ++j) x[j] = merge_mz(x[j], x[j + w]);
+    mz[k] = x[0];
   }
   // the slot's shared data is in registers: hand the slot back to the producer
   __syncwarp();
@@ -546,7 +816,7 @@ __device__ __forceinline__ bool sync_rowstats(const ScoreParams& P, ScoreCtl& ct
   unsigned long long w[4];
   if (next_unit >= 0) load_beta(P, next_unit, w);
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
+  for (int k = 0; k < kRowSets; ++k) {
     const int row = lane + 32 * k;
     if (row < n) P.partial[d.p * kMaxRows + row] = mz[k];
   }
@@ -564,16 +834,17 @@ __device__ __forceinline__ bool sync_rowstats(const ScoreParams& P, ScoreCtl& ct
 // Merge warp: fold all of a unit's (m, Z) partials into beta_r = m + log2 Z and
 // publish each row's beta with its ready tag. The partials of a unit are contiguous
 // (1 KB per item) and come in by bulk copies of up to kMergeBatch items.
-template <bool kAttn>
+template <class C>
 __device__ __forceinline__ bool merge_unit(const ScoreParams& P, ScoreCtl& ctl, const MergeJob& u,
                                            float2 (*mbuf)[kMaxRows], uint32_t& phase) {
-  constexpr int kMergeBatch = Cfg<kAttn>::kMergeBatch;
+  constexpr int kMergeBatch = C::kMergeBatch;
+  constexpr int kRowSets = C::kPartRows / 32;
   const int lane = threadIdx.x & 31;
   const int n = P.g.n_rows;
   __threadfence();
-  float M[4], Z[4];   // running (max, sum) per row, log2 units
+  float M[kRowSets], Z[kRowSets];   // running (max, sum) per row, log2 units
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
+  for (int k = 0; k < kRowSets; ++k) {
     M[k] = -INFINITY;
     Z[k] = 0.f;
   }
@@ -592,7 +863,7 @@ __device__ __forceinline__ bool merge_unit(const ScoreParams& P, ScoreCtl& ctl, 
     // all loads first (unconditional, masked afterwards), then the max, then every
     // partial rescaled to it: the loads and the exponentials are independent
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < kRowSets; ++k) {
       const int row = lane + 32 * k;
       float2 e[kMergeBatch];
 #pragma unroll
@@ -618,7 +889,7 @@ __device__ __forceinline__ bool merge_unit(const ScoreParams& P, ScoreCtl& ctl, 
     __syncwarp();
   }
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
+  for (int k = 0; k < kRowSets; ++k) {
     const int row = lane + 32 * k;
     if (row < n) {
       // one 64-bit store: a reader sees either the cleared word or (beta, 1)
@@ -680,24 +951,28 @@ __device__ __forceinline__ bool sync_colstats(const ScoreParams& P, ScoreCtl& ct
 
 // ---------------------------------------------------------------- kernel
 
-// kAttn: the window output variant (tm_v maps v; for the plain kernel tm_v is unused).
-template <bool kFull, bool kAttn>
+// kRB: 32-row blocks that hold the window rows; kFull: they are all used; kHeads: sets of rows
+// with statistics of their own; kAttn: the window output variant (tm_v maps v; for the plain
+// kernel tm_v is unused).
+template <int kRB, bool kFull, int kHeads, bool kAttn>
 __global__ void __launch_bounds__(kThreads, 1)
     score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                  const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ ScoreParams P) {
-  constexpr int kQBufs = Cfg<kAttn>::kQBufs;
-  constexpr int kKStages = Cfg<kAttn>::kKStages;
-  constexpr int kAccBufs = Cfg<kAttn>::kAccBufs;
+  using C = Cfg<kRB, kAttn>;
+  static_assert(!kAttn || (kRB == 4 && kHeads == 1), "the window output takes 128 rows");
+  constexpr int kQBufs = C::kQBufs;
+  constexpr int kKStages = C::kKStages;
+  constexpr int kAccBufs = C::kAccBufs;
   __shared__ ScoreCtl ctl;
   extern __shared__ uint8_t dyn_smem[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(dyn_smem) + 1023) & ~static_cast<uintptr_t>(1023));
-  uint8_t* qbuf = tiles;                             // kQBufs x 32 KB
-  uint8_t* kbuf = tiles + kQBufs * kTileBytes;       // kKStages x 32 KB
+  uint8_t* qbuf = tiles;                             // kQBufs Q tiles
+  uint8_t* kbuf = tiles + kQBufs * C::kQBytes;       // kKStages x 32 KB
   uint8_t* vbuf = kbuf + kKStages * kTileBytes;      // kVStages x 32 KB (window output)
   // partials being merged (bulk-copy destination, 1 KB aligned)
   float2 (*mbuf)[kMaxRows] =
-      reinterpret_cast<float2 (*)[kMaxRows]>(vbuf + Cfg<kAttn>::kVStages * kTileBytes);
+      reinterpret_cast<float2 (*)[kMaxRows]>(vbuf + C::kVStages * kTileBytes);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -718,7 +993,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&ctl.merge_empty[i], 1);
     }
     if constexpr (kAttn) {
-      for (int i = 0; i < Cfg<kAttn>::kVStages; ++i) {
+      for (int i = 0; i < C::kVStages; ++i) {
         mbar_init(&ctl.v_full[i], 1);
         mbar_init(&ctl.v_empty[i], 1);
       }
@@ -733,10 +1008,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     prefetch_tensormap(&tm_k);
     if (kAttn) prefetch_tensormap(&tm_v);
   }
-  if (threadIdx.x < kMaxRows) {
-    ctl.roww[threadIdx.x] = threadIdx.x % P.g.window;
-    ctl.rowm[threadIdx.x] = static_cast<int>(threadIdx.x) < P.g.n_rows ? 1.f : 0.f;
-  }
+  if (threadIdx.x < kMaxRows) ctl.roww[threadIdx.x] = threadIdx.x % P.g.window;
   if (warp == 1) {
     tmem_alloc(&ctl.tmem_base, kTmemCols);
     tmem_relinquish();
@@ -789,7 +1061,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           u = unit_info(P.g, item_unit(P.g, cl.p, &split));
           d.p = cl.p;
           d.unit = u.unit;
-          d.mu_off = u.mu_off;
+          d.mu_off = u.mu_off * kHeads;
           d.item0 = u.item0;
           d.phase = cl.phase;
           item_range(u, split, &d.tile0, &d.ntiles);
@@ -811,9 +1083,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           ok = false;
           break;
         }
-        mbar_arrive_expect_tx(&ctl.q_full[qb], kTileBytes);
-        tma_load_2d(qbuf + qb * kTileBytes, &tm_q, 0, static_cast<int32_t>(u.q_row0), &ctl.q_full[qb]);
-        tma_load_2d(qbuf + qb * kTileBytes + kHalfBytes, &tm_q, 64, static_cast<int32_t>(u.q_row0),
+        mbar_arrive_expect_tx(&ctl.q_full[qb], C::kQBytes);
+        tma_load_2d(qbuf + qb * C::kQBytes, &tm_q, 0, static_cast<int32_t>(u.q_row0), &ctl.q_full[qb]);
+        tma_load_2d(qbuf + qb * C::kQBytes + C::kQHalf, &tm_q, 64, static_cast<int32_t>(u.q_row0),
                     &ctl.q_full[qb]);
         q_used |= 1u << qb;
         q_last = (q_last & ~(1u << qb)) | (((qi / kQBufs) & 1u) << qb);
@@ -838,8 +1110,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           if constexpr (kAttn) {
             if (cl.phase == 1) {
               // the tile's values for the window output (streamed once, from HBM)
-              const uint32_t vs = vi % Cfg<kAttn>::kVStages;
-              const uint32_t vpar = (vi / Cfg<kAttn>::kVStages) & 1u;
+              const uint32_t vs = vi % C::kVStages;
+              const uint32_t vpar = (vi / C::kVStages) & 1u;
               if (!mbar_wait(&ctl.v_empty[vs], vpar ^ 1u, P.wait_limit_ns, &ctl.abort)) {
                 ok = false;
                 break;
@@ -864,7 +1136,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if ((q_used >> i) & 1u) mbar_wait(&ctl.q_full[i], (q_last >> i) & 1u, P.wait_limit_ns, &no_abort);
       for (int i = 0; i < kKStages; ++i)
         if ((k_used >> i) & 1u) mbar_wait(&ctl.k_full[i], (k_last >> i) & 1u, P.wait_limit_ns, &no_abort);
-      for (int i = 0; i < Cfg<kAttn>::kVStages; ++i)
+      for (int i = 0; i < C::kVStages; ++i)
         if ((v_used >> i) & 1u) mbar_wait(&ctl.v_full[i], (v_last >> i) & 1u, P.wait_limit_ns, &no_abort);
     }
   } else if (warp == 1) {
@@ -933,14 +1205,17 @@ __global__ void __launch_bounds__(kThreads, 1)
           const uint32_t d_tmem = ctl.tmem_base + ab * 128u;
           // operand roles per phase are chosen once per tile: the issue loop below is
           // branch-free (a single thread issues, so every extra instruction costs MMA rate)
-          const uint32_t qs = qaddr + qb * kTileBytes, kss = kaddr + ks * kTileBytes;
-          const uint64_t ad = sw128_desc(phase == 0 ? qs : kss);
-          const uint64_t bd = sw128_desc(phase == 0 ? kss : qs);
+          const uint32_t qs = qaddr + qb * C::kQBytes, kss = kaddr + ks * kTileBytes;
+          const bool rows_m = kRB != 1 && phase == 0;
+          const uint64_t ad = sw128_desc(rows_m ? qs : kss);
+          const uint64_t bd = sw128_desc(rows_m ? kss : qs);
+          const uint32_t idesc = rows_m ? kIdesc : idesc_bf16_f32(128, 32 * kRB);
 #pragma unroll
           for (int j = 0; j < kHeadDim / 16; ++j) {
             // the descriptor's start-address field counts 16-byte units
-            const uint64_t off = ((j >> 2) * kHalfBytes + (j & 3) * 32u) >> 4;
-            tc_mma_bf16(d_tmem, ad + off, bd + off, kIdesc, j > 0 ? 1u : 0u);
+            const uint64_t aoff = ((j >> 2) * kHalfBytes + (j & 3) * 32u) >> 4;
+            const uint64_t boff = ((j >> 2) * C::kQHalf + (j & 3) * 32u) >> 4;
+            tc_mma_bf16(d_tmem, ad + aoff, bd + boff, idesc, j > 0 ? 1u : 0u);
           }
           if (!kAttn || phase == 0) tc_commit(&ctl.k_empty[ks]);
           tc_commit(&ctl.acc_full[ab]);
@@ -954,8 +1229,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 break;
               }
               pend_ks = static_cast<int>(ks);
-              pend_vs = static_cast<int>(vi % Cfg<kAttn>::kVStages);
-              pend_vpar = (vi / Cfg<kAttn>::kVStages) & 1u;
+              pend_vs = static_cast<int>(vi % C::kVStages);
+              pend_vpar = (vi / C::kVStages) & 1u;
               pend_first = t == 0;
               ++vi;
             }
@@ -1068,7 +1343,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
         bool late_staged = false;
-        const bool last = ok && sync_rowstats(P, ctl, d, slot, next_checked ? -1 : next_unit, nslot,
+        const bool last = ok && sync_rowstats<C>(P, ctl, d, slot, next_checked ? -1 : next_unit, nslot,
                                               &late_staged);
         if (late_staged) {
           // staged after the publication: release that item now as well
@@ -1116,7 +1391,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       const MergeJob job = ctl.merge_job[ms];
       if (job.unit < 0) break;
-      if (!merge_unit<kAttn>(P, ctl, job, mbuf, mphase)) {
+      if (!merge_unit<C>(P, ctl, job, mbuf, mphase)) {
         set_error(P, ctl, 1u);
         // no bulk copy may still be writing shared memory when the CTA exits
         volatile int no_abort = 0;
@@ -1141,10 +1416,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (d.p < 0) break;
       bool ok;
       if (d.phase == 0) {
-        ok = rowstats_item<kFull, kAttn>(P, ctl, d, slot, ai);
+        if constexpr (kRB == 1)
+          ok = rowstats_by_key(P, ctl, d, slot, ai);
+        else
+          ok = rowstats_by_row<kAttn>(P, ctl, d, slot, ai);
       } else {
-        ok = warp_wait(&ctl.beta_full[slot], par, P.wait_limit_ns, &ctl.abort) &&
-             colstats_item<kFull, kAttn>(P, ctl, d, slot, ai, kbuf, oi);
+        ok = warp_wait(&ctl.beta_full[slot], par, P.wait_limit_ns, &ctl.abort);
+        if constexpr (kAttn)
+          ok = ok && colstats_with_output<kFull>(P, ctl, d, slot, ai, kbuf, oi);
+        else
+          ok = ok && colstats_by_fragment<kRB, kFull, kHeads>(P, ctl, d, slot, ai);
       }
       if (!ok) {
         set_error(P, ctl, 1u);
@@ -1185,11 +1466,11 @@ __global__ void __launch_bounds__(kHeadDim) attn_finish_kernel(const __grid_cons
   }
 }
 
-template <bool kAttn>
-cudaError_t launch_score_variant(bool full, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
-                                 const CUtensorMap& tm_v, const ScoreParams& p, int ctas, cudaStream_t stream) {
-  auto* fn = full ? score_kernel<true, kAttn> : score_kernel<false, kAttn>;
-  constexpr size_t smem = Cfg<kAttn>::kDynSmem;
+template <int kRB, bool kFull, int kHeads, bool kAttn>
+cudaError_t launch_score_variant(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
+                                 const ScoreParams& p, int ctas, cudaStream_t stream) {
+  auto* fn = score_kernel<kRB, kFull, kHeads, kAttn>;
+  constexpr size_t smem = Cfg<kRB, kAttn>::kDynSmem;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   // CTAs wait on each other's row statistics: all of them must be resident at once
@@ -1206,13 +1487,24 @@ cudaError_t launch_score_variant(bool full, const CUtensorMap& tm_q, const CUten
   return cudaLaunchKernelEx(&cfg, fn, tm_q, tm_k, tm_v, p);
 }
 
+template <int kRB>
+cudaError_t launch_score_rows(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const ScoreParams& p, int ctas,
+                              cudaStream_t stream) {
+  if (p.heads == 4) return launch_score_variant<kRB, true, 4, false>(tm_q, tm_k, tm_k, p, ctas, stream);
+  return p.g.n_rows == 32 * kRB ? launch_score_variant<kRB, true, 1, false>(tm_q, tm_k, tm_k, p, ctas, stream)
+                                : launch_score_variant<kRB, false, 1, false>(tm_q, tm_k, tm_k, p, ctas, stream);
+}
+
 }  // namespace
 
-cudaError_t launch_score(const kve_plan& plan, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
-                         const CUtensorMap* tm_v, const ScoreParams& p, int ctas, cudaStream_t stream) {
-  const bool full = plan.geo.n_rows == kMaxRows;
-  if (!tm_v) return launch_score_variant<false>(full, tm_q, tm_k, tm_k, p, ctas, stream);
-  return launch_score_variant<true>(full, tm_q, tm_k, *tm_v, p, ctas, stream);
+cudaError_t launch_score(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap* tm_v,
+                         const ScoreParams& p, int ctas, cudaStream_t stream) {
+  if (tm_v)
+    return p.g.n_rows == kMaxRows ? launch_score_variant<4, true, 1, true>(tm_q, tm_k, *tm_v, p, ctas, stream)
+                                  : launch_score_variant<4, false, 1, true>(tm_q, tm_k, *tm_v, p, ctas, stream);
+  if (p.g.n_rows <= 32) return launch_score_rows<1>(tm_q, tm_k, p, ctas, stream);
+  if (p.g.n_rows <= 64) return launch_score_rows<2>(tm_q, tm_k, p, ctas, stream);
+  return launch_score_rows<4>(tm_q, tm_k, p, ctas, stream);
 }
 
 cudaError_t launch_attn_finish(const kve_plan& plan, const float* o_part, uint16_t* o_win,
