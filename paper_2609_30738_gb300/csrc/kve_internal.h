@@ -192,6 +192,10 @@ struct kve_plan {
   kve_config cfg;
   int32_t layer_budget[kve::kMaxLayers];   // B_l per layer (all cfg.budget by default)
   kve::Geometry geo;
+  // Geometry of the score kernel: geo, or for per-query-head plans whose four query heads share
+  // a KV head's units (score_heads = 4) that of the default plan, a unit per KV head
+  kve::Geometry sgeo;
+  int32_t score_heads;
   kve::WsLayout ws;
   uint64_t wait_limit_ns;
   int32_t fault;
