@@ -82,8 +82,15 @@ int device_sms() {
 // Score items per unit for a unit of T tiles. Items hold at most kSplitTiles tiles.
 // The score kernel deals items to its CTAs round-robin, one round = one item per CTA,
 // so a split count that divides the CTA count (or is a multiple of it) makes every
-// round hold whole units; up to twice the minimum count is accepted for that.
-int32_t choose_splits(int64_t T, int64_t ctas) {
+// round hold whole units; up to twice the minimum count is accepted for that. A call of fewer
+// than kSplitTiles tiles per CTA (total_tiles over all units) takes items of total_tiles / ctas
+// tiles, so that one round gives every CTA its share: one layer of 2048 tokens (8 units of 16
+// tiles) runs on 128 CTAs instead of 16.
+int32_t choose_splits(int64_t T, int64_t ctas, int64_t total_tiles) {
+  if (ctas > 0 && total_tiles < ctas * kSplitTiles) {
+    const int64_t per_item = (total_tiles + ctas - 1) / ctas;
+    return static_cast<int32_t>((T + per_item - 1) / per_item);
+  }
   const int64_t kmin = (T + kSplitTiles - 1) / kSplitTiles;
   const int64_t kmax = std::min<int64_t>(T, 2 * kmin);
   for (int64_t k = kmin; ctas > 0 && k <= kmax; ++k)
@@ -94,10 +101,14 @@ int32_t choose_splits(int64_t T, int64_t ctas) {
 // Unit and item tables of g for its requests (req_len), units per layer and CTAs.
 void fill_units(kve::Geometry* g, int64_t ctas) {
   int64_t units = 0, items = 0;
+  int64_t total_tiles = 0;
   const int64_t units_per_req = static_cast<int64_t>(g->num_layers) * g->uheads;
   for (int r = 0; r < g->n_req; ++r) {
     g->req_tiles[r] = static_cast<int32_t>((static_cast<int64_t>(g->req_len[r]) + kTileKeys - 1) / kTileKeys);
-    g->req_splits[r] = choose_splits(g->req_tiles[r], ctas);
+    total_tiles += units_per_req * g->req_tiles[r];
+  }
+  for (int r = 0; r < g->n_req; ++r) {
+    g->req_splits[r] = choose_splits(g->req_tiles[r], ctas, total_tiles);
     g->req_unit_base[r] = units;
     g->req_item_base[r] = items;
     units += units_per_req;
