@@ -1450,20 +1450,39 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 
 // Window output, last step: O of unit u's window rows = the sum of its column items'
-// partials (fp32), written as bf16 in q_win's layout (row r of the unit at q_row0 + r).
-__global__ void __launch_bounds__(kHeadDim) attn_finish_kernel(const __grid_constant__ Geometry g,
-                                                               const float* o_part, uint16_t* o_win) {
+// partials (fp32, in item order), written as bf16 in q_win's layout (row r of the unit at
+// q_row0 + r). Bound by the partials' read (64 KB per item). A warp takes a row, 16 bytes a lane,
+// kFinishLoads items' loads in flight; a block takes kFinishRows rows, so that even one unit
+// spreads over 16 blocks: 32 layers of 8192 tokens (134 MB) take 25 us; a block per unit that
+// went through its rows and items one by one took 133.
+constexpr int kFinishRows = 8;
+constexpr int kFinishLoads = 8;
+__global__ void __launch_bounds__(kFinishRows * 32) attn_finish_kernel(const __grid_constant__ Geometry g,
+                                                                       const float* o_part, uint16_t* o_win) {
   wait_previous_kernel();   // the partials come from the score kernel launched before
   const UnitInfo u = unit_info(g, blockIdx.x);
-  const int j = threadIdx.x;   // head dimension
-  for (int r = 0; r < g.n_rows; ++r) {
-    float acc = 0.f;
-    for (int s = 0; s < u.splits; ++s)
-      acc += __ldcs(o_part + ((u.item0 + s) * kMaxRows + r) * kHeadDim + j);
-    uint32_t w;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(0.f), "f"(acc));
-    o_win[(u.q_row0 + r) * kHeadDim + j] = static_cast<uint16_t>(w & 0xFFFFu);
+  const int r = static_cast<int>(blockIdx.y) * kFinishRows + static_cast<int>(threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (r >= g.n_rows) return;
+  const float4* src = reinterpret_cast<const float4*>(o_part + (u.item0 * kMaxRows + r) * kHeadDim) + lane;
+  constexpr int64_t kStep = kMaxRows * kHeadDim / 4;   // float4 from one item to the next
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int s0 = 0; s0 < u.splits; s0 += kFinishLoads) {
+    float4 x[kFinishLoads];
+#pragma unroll
+    for (int j = 0; j < kFinishLoads; ++j)
+      if (s0 + j < u.splits) x[j] = __ldcs(src + (s0 + j) * kStep);
+#pragma unroll
+    for (int j = 0; j < kFinishLoads; ++j)
+      if (s0 + j < u.splits) {
+        acc.x += x[j].x;
+        acc.y += x[j].y;
+        acc.z += x[j].z;
+        acc.w += x[j].w;
+      }
   }
+  uint2* dst = reinterpret_cast<uint2*>(o_win + (u.q_row0 + r) * kHeadDim) + lane;
+  *dst = make_uint2(pack_bf16x2(acc.x, acc.y), pack_bf16x2(acc.z, acc.w));
 }
 
 template <int kRB, bool kFull, int kHeads, bool kAttn>
@@ -1509,8 +1528,10 @@ cudaError_t launch_score(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const
 
 cudaError_t launch_attn_finish(const kve_plan& plan, const float* o_part, uint16_t* o_win,
                                cudaStream_t stream) {
-  return launch_after_previous(attn_finish_kernel, dim3(static_cast<unsigned>(plan.geo.n_units)),
-                               dim3(kHeadDim), 0, stream, plan.geo, o_part, o_win);
+  const dim3 grid(static_cast<unsigned>(plan.geo.n_units),
+                  static_cast<unsigned>((plan.geo.n_rows + kFinishRows - 1) / kFinishRows));
+  return launch_after_previous(attn_finish_kernel, grid, dim3(kFinishRows * 32), 0, stream, plan.geo, o_part,
+                               o_win);
 }
 
 }  // namespace kve
