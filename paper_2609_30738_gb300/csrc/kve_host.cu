@@ -20,6 +20,9 @@ using kve::kMaxRows;
 using kve::kSplitTiles;
 using kve::kTileKeys;
 
+// K bytes that may stream between an item's two passes and stay in L2 (129 MB, of which the rest of
+// the traffic takes its share: two rounds of 34 MB do, three do not)
+constexpr int64_t kLagBytes = int64_t(76) << 20;
 constexpr uint64_t kDefaultWaitNs = 2000000000ull;   // 2 s
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -134,12 +137,16 @@ int32_t score_heads(const kve::Geometry& g) {
 // than the most rounds any unit's items span. Any lag at least that span is free of
 // circular waits; the extra round gives a unit's merge time to land before its first
 // phase-1 item, while the K tiles streamed in between (two rounds, about 64 MB at full
-// width) stay in L2 for the phase-1 re-read.
+// width) stay in L2 for the phase-1 re-read. Where a round's items are short (a unit length
+// whose splits divide the CTA count only with items of half the size), the merge would not have
+// landed by then, and one round more still streams no more than that: 32 layers of 20011 tokens
+// (items of 4 tiles, 20 MB a round) take 476 us of score kernel against 507.
 int32_t score_lag(const kve::Geometry& g, int64_t ctas) {
-  int64_t span = 0;
+  int64_t span = 0, tiles = 0;   // tiles: of the longest item
   const int64_t units_per_req = static_cast<int64_t>(g.num_layers) * g.uheads;
   for (int r = 0; r < g.n_req; ++r) {
     const int64_t k = g.req_splits[r];
+    tiles = std::max<int64_t>(tiles, (g.req_tiles[r] + k - 1) / k);
     // (first item) mod ctas repeats with period ctas / gcd(k, ctas) <= ctas
     const int64_t n = std::min<int64_t>(units_per_req, ctas);
     for (int64_t ul = 0; ul < n; ++ul) {
@@ -147,7 +154,8 @@ int32_t score_lag(const kve::Geometry& g, int64_t ctas) {
       span = std::max<int64_t>(span, (a + k - 1) / ctas - a / ctas);
     }
   }
-  return static_cast<int32_t>(span + 1);
+  const int64_t round_bytes = ctas * tiles * kTileKeys * kHeadDim * 2;
+  return static_cast<int32_t>(span + 1 + (3 * round_bytes <= kLagBytes ? 1 : 0));
 }
 
 }  // namespace

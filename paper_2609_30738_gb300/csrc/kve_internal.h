@@ -62,15 +62,14 @@ struct UnitInfo {
   int64_t item0;       // first score item of this unit
 };
 
-__host__ __device__ inline UnitInfo unit_info(const Geometry& g, int64_t unit) {
-  int r = 0;
-  while (r + 1 < g.n_req && g.req_unit_base[r + 1] <= unit) ++r;
+// Unit `local` (< 2^31) of request r.
+__host__ __device__ inline UnitInfo unit_at(const Geometry& g, int r, uint32_t local) {
   UnitInfo u;
-  u.unit = unit;
+  u.unit = g.req_unit_base[r] + local;
   u.r = r;
-  const int64_t local = unit - g.req_unit_base[r];
-  u.layer = static_cast<int32_t>(local / g.uheads);
-  u.h = static_cast<int32_t>(local % g.uheads);   // KV head (or query head) of the unit
+  const uint32_t uheads = static_cast<uint32_t>(g.uheads);
+  u.layer = static_cast<int32_t>(local / uheads);
+  u.h = static_cast<int32_t>(local % uheads);   // KV head (or query head) of the unit
   u.L = g.req_len[r];
   u.tiles = g.req_tiles[r];
   u.splits = g.req_splits[r];
@@ -82,29 +81,67 @@ __host__ __device__ inline UnitInfo unit_info(const Geometry& g, int64_t unit) {
   u.tok0 = g.req_tok_off[r];
   u.k_off = u.layer * g.k_sl + kvh * g.k_sh + u.tok0 * g.k_st;
   u.v_off = u.layer * g.v_sl + kvh * g.v_sh + u.tok0 * g.v_st;
-  u.mu_off = static_cast<int64_t>(g.num_layers) * g.uheads * g.req_tok_off[r] + local * u.L;
-  u.item0 = g.req_item_base[r] + local * u.splits;
+  u.mu_off = static_cast<int64_t>(g.num_layers) * g.uheads * g.req_tok_off[r] + static_cast<int64_t>(local) * u.L;
+  u.item0 = g.req_item_base[r] + static_cast<int64_t>(local) * u.splits;
   return u;
 }
 
-// Score item p (0 <= p < n_items) -> unit and split index.
-__host__ __device__ inline int64_t item_unit(const Geometry& g, int64_t p, int32_t* split) {
+__host__ __device__ inline UnitInfo unit_info(const Geometry& g, int64_t unit) {
+  int r = 0;
+  while (r + 1 < g.n_req && g.req_unit_base[r + 1] <= unit) ++r;
+  return unit_at(g, r, static_cast<uint32_t>(unit - g.req_unit_base[r]));
+}
+
+// Score item p (0 <= p < n_items) -> request, unit index within it and split index.
+struct ItemPos {
+  int32_t r;
+  uint32_t local, split;
+};
+
+__host__ __device__ inline ItemPos item_pos(const Geometry& g, int64_t p) {
   int r = 0;
   while (r + 1 < g.n_req && g.req_item_base[r + 1] <= p) ++r;
   const int64_t local = p - g.req_item_base[r];
-  *split = static_cast<int32_t>(local % g.req_splits[r]);
-  return g.req_unit_base[r] + local / g.req_splits[r];
+  return {r, static_cast<uint32_t>(local / g.req_splits[r]), static_cast<uint32_t>(local % g.req_splits[r])};
 }
 
-// Tiles [*t0, *t0 + *nt) of item `split` of unit u. The unit's tiles are cut into
-// u.splits near-equal runs; the run index is rotated by the unit index so that a
-// CTA that always holds the same split index does not always get the longer runs.
-__host__ __device__ inline void item_range(const UnitInfo& u, int split, int* t0, int* nt) {
-  const int64_t s = (split + u.local) % u.splits;
-  const int64_t a = s * u.tiles / u.splits;
-  const int64_t b = (s + 1) * u.tiles / u.splits;
-  *t0 = static_cast<int>(a);
-  *nt = static_cast<int>(b - a);
+// The item `step` items after `at`. The score kernel's producer takes every step-th item, and
+// the time it spends on one item's coordinates delays the next item's loads: 64-bit divisions
+// (about 2600 cycles an item) left the tensor cores idle for a tenth of the launch. Here one
+// 32-bit division per step, and one more where the step crosses into another request. n_items
+// stays below 2^30 (checked at planning), and so does every sum.
+__host__ __device__ inline ItemPos item_advance(const Geometry& g, ItemPos at, uint32_t step) {
+  const uint32_t units = static_cast<uint32_t>(g.num_layers * g.uheads);   // per request
+  uint32_t k = static_cast<uint32_t>(g.req_splits[at.r]);
+  const uint32_t s = at.split + step;
+  const uint32_t q = s / k;
+  at.local += q;
+  at.split = s - q * k;
+  while (at.local >= units && at.r + 1 < g.n_req) {
+    const uint32_t left = (at.local - units) * k + at.split;   // items into the next request
+    ++at.r;
+    k = static_cast<uint32_t>(g.req_splits[at.r]);
+    at.local = left / k;
+    at.split = left - at.local * k;
+  }
+  return at;
+}
+
+// Tiles [*t0, *t0 + *nt) of item `split` of the unit with index `local` in request r. The unit's
+// tiles are cut into near-equal runs; the run index is rotated by the unit index so that a CTA
+// that always holds the same split index does not always get the longer runs.
+__host__ __device__ inline void item_range(const Geometry& g, const ItemPos& at, int32_t* t0, int32_t* nt) {
+  const uint32_t k = static_cast<uint32_t>(g.req_splits[at.r]), tiles = static_cast<uint32_t>(g.req_tiles[at.r]);
+  const uint32_t s = (at.split + at.local) % k;
+  // floor(s * tiles / k) = s * (tiles / k) + floor(s * (tiles % k) / k)
+  const uint32_t whole = tiles / k, rest = tiles - whole * k;
+  const auto first = [&](uint32_t x) {
+    return x * whole + (k < 65536u ? x * rest / k
+                                   : static_cast<uint32_t>(static_cast<uint64_t>(x) * rest / k));
+  };
+  const uint32_t a = first(s), b = first(s + 1);
+  *t0 = static_cast<int32_t>(a);
+  *nt = static_cast<int32_t>(b - a);
 }
 
 // Workspace layout (byte offsets from the caller's workspace pointer).

@@ -62,13 +62,10 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Wait until the phase with the given parity has completed. Gives up (returns
-// false) when *abort becomes non-zero or limit_ns have passed. The timer is read
-// only once the barrier has been found not ready, so a wait that succeeds at once
-// costs one try_wait.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns,
-                                          volatile int* abort) {
-  if (mbar_try_wait(bar, parity)) return true;
+// The rest of mbar_wait, once the barrier has been found not ready. Out of line: the waits of
+// all roles share this code, and with it lines of the instruction cache.
+static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, uint64_t limit_ns,
+                                            volatile int* abort) {
   const uint64_t t0 = global_timer_ns();
   for (uint32_t it = 1;; ++it) {
     if (mbar_try_wait(bar, parity)) return true;
@@ -77,6 +74,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64
       if (global_timer_ns() - t0 > limit_ns) return false;
     }
   }
+}
+
+// Wait until the phase with the given parity has completed. Gives up (returns
+// false) when *abort becomes non-zero or limit_ns have passed. The timer is read
+// only once the barrier has been found not ready, so a wait that succeeds at once
+// costs one try_wait.
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns,
+                                          volatile int* abort) {
+  return mbar_try_wait(bar, parity) || mbar_wait_slow(bar, parity, limit_ns, abort);
 }
 
 // Two waits whose first polls are issued together, so that their latencies overlap when
@@ -253,6 +259,13 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
       : "r"(taddr));
 #pragma unroll
   for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+}
+
+// One fp32 column of this warp's 32 TMEM lanes.
+__device__ __forceinline__ float tmem_ld1(uint32_t taddr) {
+  uint32_t r;
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr));
+  return __uint_as_float(r);
 }
 
 // Fragment loads of 16 TMEM lanes (taddr's lane and the 15 after it; the first or second

@@ -69,8 +69,13 @@ constexpr uint32_t kIdescMN = kIdesc | (1u << 15) | (1u << 16);
 constexpr uint32_t kMNLbo = kHalfBytes;
 constexpr uint32_t kMNSbo = 1024;
 
-// Pipeline depths of the two variants. The plain kernel: 2 Q buffers, 3 K stages, 4
-// score accumulators, partials merged 40 per bulk copy. With the window output (kAttn)
+// Pipeline depths of the two variants. The plain kernel: 2 Q buffers, 4 K stages, 4
+// score accumulators, a merge buffer of 20 partials. A K stage's turn is its load (1700 to 2200
+// cycles under load), its MMAs (600) and its release (450), 1100 cycles a tile over three stages;
+// the fourth takes half of the 40-partial buffer that a unit of 38 items filled in one copy (see
+// merge_unit). Together with the 32-bit item coordinates (item_advance), at 32 layers: given
+// normalisers 338 -> 326 us at 32768 tokens and 227 -> 208 at 20011 (the HBM time is 328 and 205),
+// both passes 601 -> 571 over requests of 4099, 9473 and 16001 tokens. With the window output (kAttn)
 // the column pass also streams V and accumulates O^T on the tensor cores: a column
 // tile's K stage holds its probabilities P^T until the O^T MMA has read them, so the
 // shared memory goes to 3 K stages and 2 V stages with a single Q buffer and a merge
@@ -86,10 +91,10 @@ struct Cfg {
   static constexpr uint32_t kQHalf = kQRows * 128u;          // one 64-element column block of Q
   static constexpr uint32_t kQBytes = 2 * kQHalf;
   static constexpr int kQBufs = kAttn ? 1 : 2;
-  static constexpr int kKStages = kRB == 1 ? 4 : 3;
+  static constexpr int kKStages = kAttn ? 3 : 4;
   static constexpr int kVStages = kAttn ? 2 : 0;
   static constexpr int kAccBufs = kAttn ? 3 : 4;
-  static constexpr int kMergeBatch = kAttn ? 16 : 40;   // partials per bulk copy (1 KB each)
+  static constexpr int kMergeBatch = kAttn ? 16 : 20;   // partials per bulk copy (1 KB each)
   static constexpr size_t kMergeBytes = static_cast<size_t>(kMergeBatch) * kMaxRows * sizeof(float2);
   static constexpr size_t kDynSmem =
       kQBufs * kQBytes + (kKStages + kVStages) * kTileBytes + kMergeBytes + 1024;
@@ -831,71 +836,92 @@ __device__ __forceinline__ bool sync_rowstats(const ScoreParams& P, ScoreCtl& ct
   return __shfl_sync(0xffffffffu, last, 0) != 0;
 }
 
-// Merge warp: fold all of a unit's (m, Z) partials into beta_r = m + log2 Z and
-// publish each row's beta with its ready tag. The partials of a unit are contiguous
-// (1 KB per item) and come in by bulk copies of up to kMergeBatch items.
+// Fold N partials' (m, Z) of a lane's four rows (e[j] = {row 0, row 1}, {row 2, row 3}) into the
+// running (max, sum), log2 units: the max first, then every partial rescaled to it, so that
+// the exponentials are independent. Absent partials are (-inf, 0).
+template <int N>
+__device__ __forceinline__ void fold_partials(const float4 (&e)[N][2], float (&M)[4], float (&Z)[4]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const auto part = [&](int j) {
+      const float4 x = e[j][k >> 1];
+      return k & 1 ? make_float2(x.z, x.w) : make_float2(x.x, x.y);
+    };
+    float mb = M[k];
+#pragma unroll
+    for (int j = 0; j < N; ++j) mb = fmaxf(mb, part(j).x);
+    const float ref = mb == -INFINITY ? 0.f : mb;   // no key seen yet: every term below is 0
+    float z0 = Z[k] * ex2(M[k] - ref), z1 = 0.f;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const float t = part(j).y;
+      if (j & 1) z1 = fmaf(t, ex2(part(j).x - ref), z1); else z0 = fmaf(t, ex2(part(j).x - ref), z0);
+    }
+    M[k] = mb;
+    Z[k] = z0 + z1;
+  }
+}
+
+// Merge warp: fold all of a unit's (m, Z) partials into beta_r = m + log2 Z and publish each
+// row's beta with its ready tag; a lane has rows 4 lane .. 4 lane + 3. The partials (1 KB per
+// item) come from L2 by two ways at once: up to kMergeBatch by a bulk copy into shared memory,
+// and up to kMergeDirect into registers, so that a unit of 38 items takes about one copy's
+// latency with half the buffer (whose other half is part of the fourth K stage).
+constexpr int kMergeDirect = 18, kMergeFold = 10;
 template <class C>
 __device__ __forceinline__ bool merge_unit(const ScoreParams& P, ScoreCtl& ctl, const MergeJob& u,
                                            float2 (*mbuf)[kMaxRows], uint32_t& phase) {
-  constexpr int kMergeBatch = C::kMergeBatch;
-  constexpr int kRowSets = C::kPartRows / 32;
   const int lane = threadIdx.x & 31;
   const int n = P.g.n_rows;
   __threadfence();
-  float M[kRowSets], Z[kRowSets];   // running (max, sum) per row, log2 units
+  float M[4], Z[4];
 #pragma unroll
-  for (int k = 0; k < kRowSets; ++k) {
+  for (int k = 0; k < 4; ++k) {
     M[k] = -INFINITY;
     Z[k] = 0.f;
   }
-  for (int s0 = 0; s0 < u.splits; s0 += kMergeBatch) {
-    const int cnt = u.splits - s0 < kMergeBatch ? u.splits - s0 : kMergeBatch;
+  constexpr int kRowF4 = kMaxRows / 2;   // float4 per partial
+  const float4 none = make_float4(-INFINITY, 0.f, -INFINITY, 0.f);
+  for (int s0 = 0; s0 < u.splits; s0 += C::kMergeBatch + kMergeDirect) {
+    const int bulk = u.splits - s0 < C::kMergeBatch ? u.splits - s0 : C::kMergeBatch;
     if (lane == 0) {
-      // the other CTAs' partials (acquired above) and this warp's reads of the
-      // previous batch come before the copy
+      // the other CTAs' partials (acquired above) and this warp's reads of the previous
+      // batch come before the copy
       fence_proxy_async();
-      const uint32_t bytes = static_cast<uint32_t>(cnt) * kMaxRows * sizeof(float2);
+      const uint32_t bytes = static_cast<uint32_t>(bulk) * kMaxRows * sizeof(float2);
       mbar_arrive_expect_tx(&ctl.merge_bar, bytes);
       bulk_load(&mbuf[0][0], &P.partial[(u.item0 + s0) * kMaxRows], bytes, &ctl.merge_bar);
     }
+    if (const int d0 = s0 + bulk; d0 < u.splits) {
+      const float4* src = reinterpret_cast<const float4*>(P.partial + (u.item0 + d0) * kMaxRows) + 2 * lane;
+      float4 e[kMergeDirect][2];
+#pragma unroll
+      for (int j = 0; j < kMergeDirect; ++j)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) e[j][q] = d0 + j < u.splits ? __ldcg(src + j * kRowF4 + q) : none;
+      fold_partials(e, M, Z);
+    }
     if (!warp_wait(&ctl.merge_bar, phase, P.wait_limit_ns, &ctl.abort)) return false;
     phase ^= 1u;
-    // all loads first (unconditional, masked afterwards), then the max, then every
-    // partial rescaled to it: the loads and the exponentials are independent
+#pragma unroll 1
+    for (int d0 = 0; d0 < bulk; d0 += kMergeFold) {
+      float4 e[kMergeFold][2];
 #pragma unroll
-    for (int k = 0; k < kRowSets; ++k) {
-      const int row = lane + 32 * k;
-      float2 e[kMergeBatch];
+      for (int j = 0; j < kMergeFold; ++j)
 #pragma unroll
-      for (int j = 0; j < kMergeBatch; ++j) {
-        const float2 x = mbuf[j][row];
-        e[j] = j < cnt ? x : make_float2(-INFINITY, 0.f);
-      }
-      float mb = M[k];
-#pragma unroll
-      for (int j = 0; j < kMergeBatch; ++j) mb = fmaxf(mb, e[j].x);
-      if (row >= n || mb == -INFINITY) continue;
-      float z0 = M[k] == -INFINITY ? 0.f : Z[k] * ex2(M[k] - mb), z1 = 0.f, z2 = 0.f, z3 = 0.f;
-#pragma unroll
-      for (int j = 0; j < kMergeBatch; j += 4) {
-        z0 = fmaf(e[j].y, ex2(e[j].x - mb), z0);   // ex2(-inf) = 0 for empty partials
-        if (j + 1 < kMergeBatch) z1 = fmaf(e[j + 1].y, ex2(e[j + 1].x - mb), z1);
-        if (j + 2 < kMergeBatch) z2 = fmaf(e[j + 2].y, ex2(e[j + 2].x - mb), z2);
-        if (j + 3 < kMergeBatch) z3 = fmaf(e[j + 3].y, ex2(e[j + 3].x - mb), z3);
-      }
-      M[k] = mb;
-      Z[k] = (z0 + z1) + (z2 + z3);
+        for (int q = 0; q < 2; ++q)
+          e[j][q] = d0 + j < bulk ? reinterpret_cast<const float4*>(mbuf[d0 + j])[2 * lane + q] : none;
+      fold_partials(e, M, Z);
     }
     __syncwarp();
   }
 #pragma unroll
-  for (int k = 0; k < kRowSets; ++k) {
-    const int row = lane + 32 * k;
+  for (int k = 0; k < 4; ++k) {
+    const int row = 4 * lane + k;
     if (row < n) {
       // one 64-bit store: a reader sees either the cleared word or (beta, 1)
-      const float b = M[k] + lg2(Z[k]);
       const unsigned long long word =
-          (1ull << 32) | static_cast<unsigned long long>(__float_as_uint(b));
+          (1ull << 32) | static_cast<unsigned long long>(__float_as_uint(M[k] + lg2(Z[k])));
       __stcg(&P.beta[u.unit * kMaxRows + row], word);
     }
   }
@@ -1031,6 +1057,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int64_t G = gridDim.x;
       const int64_t own = (n1 - blockIdx.x + G - 1) / G;
       int64_t jr = 0, jc = 0;
+      ItemPos row_at = item_pos(P.g, blockIdx.x), col_at = row_at;   // items jr and jc
       for (;;) {
         Claim cl;
         bool have = true;
@@ -1057,14 +1084,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         ItemDesc d;
         UnitInfo u;
         if (have) {
-          int split;
-          u = unit_info(P.g, item_unit(P.g, cl.p, &split));
+          const ItemPos at = cl.phase == 0 ? row_at : col_at;
+          const ItemPos next = item_advance(P.g, at, gridDim.x);
+          if (cl.phase == 0) row_at = next; else col_at = next;
+          u = unit_at(P.g, at.r, at.local);
           d.p = cl.p;
           d.unit = u.unit;
           d.mu_off = u.mu_off * kHeads;
           d.item0 = u.item0;
           d.phase = cl.phase;
-          item_range(u, split, &d.tile0, &d.ntiles);
+          item_range(P.g, at, &d.tile0, &d.ntiles);
           d.L = u.L;
           d.splits = u.splits;
           d.tok0 = static_cast<int32_t>(u.tok0);
