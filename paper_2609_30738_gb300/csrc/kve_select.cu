@@ -16,7 +16,9 @@
 //     at 0);
 //  5. write the admitted positions ascending (and optionally in admission order,
 //     with the best-minus-second margin of every admission).
-// The block has one thread per pool slot (256 for C <= 256, else 512). A launch for
+// The block has one thread per pool slot (256 for C <= 256, else 512). Up to 256 slots every
+// pair's dot product is formed before the greedy, on tcgen05 (gram_greedy); beyond that each
+// admission forms its own 512 dots. A launch for
 // several coefficient profiles (Section 3.3 re-selects for every profile a search
 // tries; mu and sigma do not depend on them) runs one CTA per (unit, profile), the
 // profile's coefficients and scratch taken from a table in the kernel parameters.
@@ -68,8 +70,22 @@ __device__ __forceinline__ float unord_key(uint32_t k) {
   return __uint_as_float(u);
 }
 
+// Dot products of a pool of up to 256 keys, held for the greedy: the slots in two halves H0, H1
+// of 128, G00 = H0 H0^T and G11 = H1 H1^T in TMEM (256 columns: column j holds the dots with
+// slot j of the lane's own half), G01 = H0 H1^T in shared memory, row-major with an odd pitch so
+// that a row and a column are both read without bank conflicts.
+constexpr uint32_t kGramCols = 256;
+constexpr int kGramPitch = 129;
+constexpr uint32_t kGramHalf = 128 * kHeadDim * 2;   // staged keys of one half: two 64-dim blocks
+constexpr uint64_t kGramWaitNs = 2000000000ull;
+
 template <int NT>
 struct SelSmall {
+  uint64_t gram_bar[3];          // G01, G11, G00 formed
+  uint4 win[2][2];               // per warp of the greedy: best keys and tie keys, by step parity
+  uint32_t wsec[2][4];           // and second keys
+  uint32_t tmem;
+  volatile int abort;            // never set: the waits here have no other party
   uint32_t warp_tot[NT / 32];
   uint32_t red[2][NT / 32][4];   // per warp: best key, best slot, second key
   uint32_t prefix, need, cnt, maxkey, teq, ncand;
@@ -126,7 +142,7 @@ __device__ __forceinline__ uint32_t block_excl_suffix(uint32_t x, SelSmall<NT>& 
 
 // Step 4 in the selection's CTA (P.k_out set): unit u's compact cache [B + W][d] as the
 // gather kernel writes it. Rows r < nvalid are the kept candidates in ascending position
-// (rpos[r]; their key rows are still staged in shared memory, row rslot[r]); rows
+// (rpos[r]; krow != null: their key rows are still staged in shared memory, row rslot[r]); rows
 // m .. m+W-1 are the window tokens Lc .. L-1; every other row is zero. A half-warp
 // copies a 256-byte row with 16-byte accesses; all loads of a batch are in flight before
 // its first store. The copy is bit-exact.
@@ -153,7 +169,8 @@ __device__ __forceinline__ void write_compact_cache(const SelectParams& P, const
       if (r < nvalid) {
         const int s = rpos[r];
         if (s >= 0 && s < Lc) {                      // never read outside the unit
-          kv[p] = krow[rslot[r] * kRowChunks + lane16];
+          kv[p] = krow ? krow[rslot[r] * kRowChunks + lane16]
+                       : __ldcg(reinterpret_cast<const uint4*>(ksrc + s * P.g.k_st) + lane16);
           vv[p] = __ldcs(reinterpret_cast<const uint4*>(vsrc + s * P.g.v_st) + lane16);
         }
       } else if (r >= m && r < m + W) {
@@ -173,6 +190,152 @@ __device__ __forceinline__ void write_compact_cache(const SelectParams& P, const
   }
 }
 
+// Address of 16-byte chunk c of staged key row r in the tcgen05 operand layout: halves of 128
+// rows, each two blocks of 64 dims (128-byte rows, 128-byte swizzle).
+__device__ __forceinline__ uint8_t* gram_chunk(uint8_t* keys, int r, int c) {
+  return keys + (r >> 7) * kGramHalf + (c >> 3) * (kGramHalf / 2) + (r & 127) * 128 + (((c ^ r) & 7) << 4);
+}
+
+// All dot products of the staged pool (n_half halves of 128 rows at `keys`, 1 KB aligned; rows
+// past the pool hold anything): G00 and G11 into TMEM, G01 over the staged keys. False if a
+// bounded wait ran out (block-uniform). Every thread calls it after a block barrier.
+template <int NT>
+__device__ __forceinline__ bool gram_form(SelSmall<NT>& sh, uint8_t* keys, int n_half) {
+  static_assert(NT == 256, "two warps per TMEM lane quadrant");
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t tmem = sh.tmem;
+  const uint32_t base = smem_u32(keys);
+  auto product = [&](int a, int b, uint32_t col, uint64_t* bar) {
+    const uint64_t ad = sw128_desc(base + a * kGramHalf), bd = sw128_desc(base + b * kGramHalf);
+#pragma unroll
+    for (int j = 0; j < kHeadDim / 16; ++j) {
+      const uint64_t off = ((j >> 2) * (kGramHalf / 2) + (j & 3) * 32u) >> 4;
+      tc_mma_bf16(tmem + col, ad + off, bd + off, idesc_bf16_f32(128, 128), j > 0 ? 1u : 0u);
+    }
+    tc_commit(bar);
+  };
+  auto wait = [&](int i) { return mbar_wait(&sh.gram_bar[i], 0u, kGramWaitNs, &sh.abort); };
+  // after a wait that ran out: the products under way are waited for once more
+  auto give_up = [&](int first, int last) {
+    if (threadIdx.x == 0)
+      for (int i = first; i <= last; ++i) wait(i);
+    __syncthreads();
+    return false;
+  };
+  bool ok = true;
+  if (n_half == 1) {
+    if (threadIdx.x == 0) product(0, 0, 0u, &sh.gram_bar[2]);
+    __syncwarp();
+    ok = wait(2);
+    tc_fence_after();
+    return __syncthreads_and(ok) != 0 || give_up(2, 2);
+  }
+  // G01 goes through G00's columns to registers, and over the keys once nothing reads them
+  if (threadIdx.x == 0) {
+    product(0, 1, 0u, &sh.gram_bar[0]);
+    product(1, 1, 128u, &sh.gram_bar[1]);
+  }
+  __syncwarp();
+  ok = wait(0);
+  tc_fence_after();
+  float v[2][32];
+  const uint32_t src = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + 64u * (warp >> 2);
+  tmem_ld32(src, v[0]);
+  tmem_ld32(src + 32u, v[1]);
+  tmem_wait_ld(v[0]);
+  tmem_wait_ld(v[1]);
+  tc_fence_before();
+  ok = __syncthreads_and(ok) != 0;
+  if (!ok) return give_up(0, 1);
+  tc_fence_after();
+  if (threadIdx.x == 0) product(0, 0, 0u, &sh.gram_bar[2]);
+  __syncwarp();
+  ok = wait(1) && wait(2);
+  tc_fence_after();
+  if (__syncthreads_and(ok) == 0) return give_up(0, 2);
+  float* dst = reinterpret_cast<float*>(keys) + ((warp & 3) * 32 + lane) * kGramPitch + 64 * (warp >> 2);
+#pragma unroll
+  for (int j = 0; j < 32; ++j) dst[j] = v[0][j];
+#pragma unroll
+  for (int j = 0; j < 32; ++j) dst[32 + j] = v[1][j];
+  __syncthreads();
+  return true;
+}
+
+// The greedy over a pool of up to 256 slots whose dot products stand (gram_form): warps 0 .. 3,
+// thread i owns slots i and 128 + i. A step is a chain of latencies -- two warp reductions, one
+// barrier of the four warps, the fold of their results -- after which the admitted slot's dots
+// are one TMEM column and one shared-memory row or column: 0.29 us, against 0.53 us with the dots
+// of every admission formed when it is known (16 mma.sync per warp, whose 8 columns all held the
+// same key). 64 admissions: 18.7 us per unit and 2.5 us for the products, against 33.8; a launch
+// of 256 units of 8192 tokens 44.6 us against 58.5, of 32768 tokens 72.1 against 82. st[], inv: normalised base score and inverse norm of the thread's slots (inactive
+// slots: `active` false); tie: position << 9 | slot or the slot.
+struct GreedySlot {
+  float st, inv, corr;
+  uint32_t tie;
+  bool active;
+};
+template <int NT, class Admit>
+__device__ __forceinline__ void gram_greedy(SelSmall<NT>& sh, const float* g01, const float* inv, GreedySlot (&s)[2],
+                                            float lambda2, int nsel, bool packed, bool want_second, Admit admit) {
+  const int i = threadIdx.x, warp = i >> 5, lane = i & 31;
+  const uint32_t tcol = sh.tmem + (static_cast<uint32_t>(warp * 32) << 16);
+  for (int t = 0; t < nsel; ++t) {
+    uint32_t k[2], q[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      k[e] = s[e].active ? ord_key(fmaf(lambda2, s[e].corr, s[e].st)) : 0u;
+      q[e] = s[e].active ? s[e].tie : 0xFFFFFFFFu;
+    }
+    const bool second = k[1] > k[0] || (k[1] == k[0] && q[1] < q[0]);
+    const uint32_t key = second ? k[1] : k[0], tie = second ? q[1] : q[0];
+    const uint32_t wmax = __reduce_max_sync(0xffffffffu, key);
+    const uint32_t holders = __ballot_sync(0xffffffffu, key == wmax);
+    uint32_t wtie = tie;   // of the only holder, or the smallest
+    if (holders & (holders - 1u)) wtie = __reduce_min_sync(0xffffffffu, key == wmax ? tie : 0xFFFFFFFFu);
+    const bool mine = key == wmax && tie == wtie;
+    if (mine) {
+      reinterpret_cast<uint32_t*>(&sh.win[t & 1][0])[warp] = key;
+      reinterpret_cast<uint32_t*>(&sh.win[t & 1][1])[warp] = tie;
+    }
+    if (want_second) {
+      const uint32_t wsec = __reduce_max_sync(0xffffffffu, mine ? (second ? k[0] : k[1]) : key);
+      if (lane == 0) sh.wsec[t & 1][warp] = wsec;
+    }
+    named_bar_sync(1, 128);
+    const uint4 wk = sh.win[t & 1][0], wt = sh.win[t & 1][1];
+    // the largest key, then the smallest tie key
+    const bool b01 = wk.y > wk.x || (wk.y == wk.x && wt.y < wt.x), b23 = wk.w > wk.z || (wk.w == wk.z && wt.w < wt.z);
+    const uint32_t ka = b01 ? wk.y : wk.x, ta = b01 ? wt.y : wt.x, kb = b23 ? wk.w : wk.z, tb = b23 ? wt.w : wt.z;
+    const bool b = kb > ka || (kb == ka && tb < ta);
+    const uint32_t best = b ? kb : ka, btie = b ? tb : ta;
+    const int js = static_cast<int>((packed ? (btie & 511u) : btie) & (kGramCols - 1u));
+    const int jj = js & 127;
+    // the dots with slot js: within its half in TMEM (column js), across in g01
+    const float tm = tmem_ld1(tcol + static_cast<uint32_t>(js));
+    const float of = js < 128 ? g01[jj * kGramPitch + i] : g01[i * kGramPitch + jj];
+    const float inv_j = inv[js];
+    if (i == 0) {
+      uint32_t sec = 0u;
+      if (want_second) {
+        // runner-up: the other warps' best and the winning warp's second
+        const int w = b ? (b23 ? 3 : 2) : (b01 ? 1 : 0);
+        const uint32_t all[4] = {wk.x, wk.y, wk.z, wk.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sec = max(sec, e == w ? sh.wsec[t & 1][e] : all[e]);
+      }
+      admit(t, js, btie, best, sec);
+    }
+    if (i == jj) {
+      if (js < 128) s[0].active = false; else s[1].active = false;
+    }
+    tmem_wait_ld();
+    const float d0 = js < 128 ? tm : of, d1 = js < 128 ? of : tm;
+    s[0].corr = fmaxf(s[0].corr, d0 * s[0].inv * inv_j);
+    s[1].corr = fmaxf(s[1].corr, d1 * s[1].inv * inv_j);
+  }
+}
+
 // The coefficients of one selection: those of SelectParams (kMulti = false), or
 // profile first + blockIdx.y of a table (kMulti = true).
 struct OneProfile {
@@ -182,11 +345,33 @@ struct OneProfile {
 template <int NT, class Prof>
 __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __grid_constant__ SelectParams P,
                                                     const __grid_constant__ Prof prof) {
+  constexpr bool kGram = NT == 256;   // the dots of every pair of the pool before the greedy
   __shared__ SelSmall<NT> sh;
-  extern __shared__ __align__(16) uint8_t dyn[];
-  wait_previous_kernel();   // mu and sigma come from the score kernel launched before
+  extern __shared__ __align__(16) uint8_t dyn_smem[];
+  // (the staged keys are tcgen05 operands there: 1 KB aligned)
+  uint8_t* dyn = kGram ? reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dyn_smem) + 1023) &
+                                                     ~static_cast<uintptr_t>(1023))
+                       : dyn_smem;
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
+  if constexpr (kGram) {
+    // Allocated and relinquished first thing: the SM starts no second block of the kernel before
+    // this block has given up its right to allocate (measured: half the blocks of a 256-unit
+    // launch began 44 us late when this stood before the greedy).
+    if (warp == 0) {
+      tmem_alloc(&sh.tmem, kGramCols);
+      tmem_relinquish();
+    }
+    if (tid == 0) {
+      for (int i = 0; i < 3; ++i) mbar_init(&sh.gram_bar[i], 1);
+      sh.abort = 0;
+      fence_mbar_init();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+  }
+  wait_previous_kernel();   // mu and sigma come from the score kernel launched before
 
   const UnitInfo u = unit_info(P.g, blockIdx.x);
   const int W = P.g.window;
@@ -571,8 +756,8 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
   // exactly C positions (the pool writes above are bounded by the pool's size all the
   // same). Should that ever fail, the pool would hold unwritten slots: the unit is then
   // reported through the error word and gets no selection.
-  if (n_above + needT != static_cast<uint32_t>(C) || needT > n_eq || needT == 0u) {
-    if (tid == 0 && P.err) atomicOr(P.err, kErrCheck);
+  auto no_selection = [&](uint32_t why) {
+    if (tid == 0 && P.err) atomicOr(P.err, why);
     int32_t* out = P.indices + out_off + u.unit * B;
     for (int r = tid; r < B; r += NT) out[r] = -1;
     if (P.order)
@@ -580,6 +765,12 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
     if (P.margins)
       for (int r = tid; r < B; r += NT) P.margins[out_off + u.unit * B + r] = 0.f;
     if (P.k_out) write_compact_cache<NT>(P, u, Lc, nsel, 0, nullptr, nullptr, nullptr);
+  };
+  if (n_above + needT != static_cast<uint32_t>(C) || needT > n_eq || needT == 0u) {
+    no_selection(kErrCheck);
+    if constexpr (kGram) {
+      if (warp == 0) tmem_dealloc(sh.tmem, kGramCols);
+    }
     return;
   }
   if (n_eq <= kTieCap) {
@@ -652,9 +843,80 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
 #pragma unroll
     for (int q = 0; q < kRows; ++q) {
       const int r = (q * (NT / 32) + warp) * 2 + (lane >> 4);
-      if (r < C) krow[r * kRowChunks + (lane & 15)] = xr[q];
+      if (r < C) {
+        if constexpr (kGram)
+          *reinterpret_cast<uint4*>(gram_chunk(big, r, lane & 15)) = xr[q];
+        else
+          krow[r * kRowChunks + (lane & 15)] = xr[q];
+      }
     }
   }
+  int32_t* order = P.order ? P.order + out_off + u.unit * B : nullptr;
+  float* margins = P.margins ? P.margins + out_off + u.unit * B : nullptr;
+  // admitted positions in admission order (the pool's other pair of arrays is free),
+  // and their slots when the compact cache is written here
+  int32_t* adm = packed ? spos : cpos;
+  int32_t* adm_slot = reinterpret_cast<int32_t*>(packed ? skey : ckey);
+  // the inverse norm of a staged row: its squares summed in two chains
+  auto row_inv_norm = [](auto chunk) {
+    float ss0 = 0.f, ss1 = 0.f;
+#pragma unroll 4
+    for (int c = 0; c < kChunks; ++c) {
+      const uint4 w = chunk(c);
+      const uint32_t w4[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float lo = __uint_as_float(w4[e] << 16);
+        const float hi = __uint_as_float(w4[e] & 0xFFFF0000u);
+        ss0 = fmaf(lo, lo, ss0);
+        ss1 = fmaf(hi, hi, ss1);
+      }
+    }
+    const float ss = ss0 + ss1;
+    return ss > 0.f ? inv_sqrt(ss) : 0.f;
+  };
+  const auto tie_key = [&](int slot) {
+    return packed ? (static_cast<uint32_t>(ppos[slot]) << 9) | static_cast<uint32_t>(slot) : static_cast<uint32_t>(slot);
+  };
+  if constexpr (kGram) {
+    // 5. greedy admissions on the pool's dot products
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the keys are read by the MMAs
+    __syncthreads();
+    // a slot's inverse norm from its own staged row
+    if (tid < C) inv[tid] = row_inv_norm([&](int c) { return *reinterpret_cast<const uint4*>(gram_chunk(big, tid, c)); });
+    __syncthreads();
+    const bool formed = gram_form<NT>(sh, big, C > 128 ? 2 : 1);
+    if (formed && warp < 4) {
+      GreedySlot s[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int slot = tid + 128 * e;
+        s[e].active = slot < C;
+        s[e].st = s[e].active ? __fdiv_rn(unord_key(pkey[slot]), smax) : 0.f;
+        s[e].inv = s[e].active ? inv[slot] : 0.f;
+        s[e].corr = 0.f;
+        s[e].tie = s[e].active ? tie_key(slot) : 0xFFFFFFFFu;
+      }
+      gram_greedy<NT>(sh, reinterpret_cast<const float*>(big), inv, s, lambda2, nsel, packed, margins != nullptr,
+                      [&](int t, int js, uint32_t btie, uint32_t best, uint32_t sec) {
+                        const int pos = packed ? static_cast<int>(btie >> 9) : ppos[js];
+                        adm[t] = pos;
+                        adm_slot[t] = js;
+                        if (order) order[t] = pos;
+                        if (margins) margins[t] = sec ? unord_key(best) - unord_key(sec) : INFINITY;
+                      });
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+      tc_fence_after();
+      tmem_dealloc(sh.tmem, kGramCols);
+    }
+    if (!formed) {
+      no_selection(kErrWait);
+      return;
+    }
+  } else {
   __syncthreads();
 
   // 5. greedy admissions. Lane (g, t) of a warp owns slot
@@ -673,27 +935,10 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
   // from inv[] after the first barrier of the loop below)
   float my_inv = 0.f;
   if (active) {
-    const uint4* row = krow + slot * kRowChunks;
-    float ss0 = 0.f, ss1 = 0.f;
-#pragma unroll 4
-    for (int c = 0; c < kChunks; ++c) {
-      const uint4 w = row[c];
-      const uint32_t w4[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float lo = __uint_as_float(w4[e] << 16);
-        const float hi = __uint_as_float(w4[e] & 0xFFFF0000u);
-        ss0 = fmaf(lo, lo, ss0);
-        ss1 = fmaf(hi, hi, ss1);
-      }
-    }
-    const float ss = ss0 + ss1;
-    my_inv = ss > 0.f ? inv_sqrt(ss) : 0.f;
+    my_inv = row_inv_norm([&](int c) { return krow[slot * kRowChunks + c]; });
     inv[slot] = my_inv;
   }
-  const uint32_t my_tie = !active ? 0xFFFFFFFFu
-                                  : (packed ? (static_cast<uint32_t>(ppos[slot]) << 9) | static_cast<uint32_t>(slot)
-                                            : static_cast<uint32_t>(slot));
+  const uint32_t my_tie = active ? tie_key(slot) : 0xFFFFFFFFu;
   const uint32_t* kw = reinterpret_cast<const uint32_t*>(krow);   // 4 * kRowChunks words per row
   uint32_t afr[2][8][4];
 #pragma unroll
@@ -707,12 +952,6 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
       afr[m][s8][3] = r1 < C ? kw[r1 * kRowWords + 8 * s8 + tq + 4] : 0u;
     }
   }
-  int32_t* order = P.order ? P.order + out_off + u.unit * B : nullptr;
-  float* margins = P.margins ? P.margins + out_off + u.unit * B : nullptr;
-  // admitted positions in admission order (the pool's other pair of arrays is free),
-  // and their slots when the compact cache is written here
-  int32_t* adm = packed ? spos : cpos;
-  int32_t* adm_slot = reinterpret_cast<int32_t*>(packed ? skey : ckey);
   for (int t = 0; t < nsel; ++t) {
     const uint32_t key = active ? ord_key(fmaf(lambda2, corr, my_st)) : 0u;
     const uint32_t wmax = __reduce_max_sync(0xffffffffu, key);
@@ -787,6 +1026,7 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
     const float dot = (tq >> 1) ? dhi : dlo;
     if (active) corr = fmaxf(corr, dot * my_inv * inv[js]);
   }
+  }   // (!kGram)
 
   // 6. admitted positions in ascending order (rank among the nsel admissions), then -1
   __syncthreads();
@@ -812,7 +1052,7 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
     for (int r = nsel + tid; r < B; r += NT) margins[r] = 0.f;
   if (P.k_out) {
     __syncthreads();
-    write_compact_cache<NT>(P, u, Lc, nsel, nsel, rpos, rslot, krow);
+    write_compact_cache<NT>(P, u, Lc, nsel, nsel, rpos, rslot, kGram ? nullptr : krow);
   }
 }
 
@@ -820,12 +1060,16 @@ template <int NT>
 constexpr size_t select_smem() {
   // candidate keys (also reused for the pooling tiles, the histograms, the threshold
   // bin's keys and the tie list) + 5 arrays + the first-digit histogram
-  return kRowChunks * NT * sizeof(uint4) + 5 * NT * sizeof(int32_t) + kBins * sizeof(uint32_t);
+  // (+ 1 KB: alignment of the keys as tcgen05 operands)
+  return kRowChunks * NT * sizeof(uint4) + 5 * NT * sizeof(int32_t) + kBins * sizeof(uint32_t) +
+         (NT == 256 ? 1024 : 0);
 }
 static_assert(kRowChunks * 256 * sizeof(uint4) >= kBins * sizeof(uint32_t), "histogram fits");
 static_assert(kRowChunks * 256 * sizeof(uint4) >= 2 * (256 * kPoolRun * kPoolRuns + 256) * sizeof(float),
               "pool tiles fit");
 static_assert(kRowChunks * 256 * sizeof(uint4) >= kTieCap * sizeof(int32_t), "tie list fits");
+static_assert(kRowChunks * 256 * sizeof(uint4) >= 128 * kGramPitch * sizeof(float) &&
+              kRowChunks * 256 * sizeof(uint4) >= 2 * kGramHalf, "staged keys and their dots fit");
 static_assert(2 * kMaxPoolCand <= kBins, "ranked positions and rows fit the first-digit histogram's place");
 // both parameter blocks of a multi-profile launch fit the 32764-byte kernel
 // parameter space

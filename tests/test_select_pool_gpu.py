@@ -1,0 +1,74 @@
+"""Pool sizes at the edges of the selector's greedy: one half of 128 slots and two, a slot short of a
+half and one past it, the largest pool whose dot products stand before the greedy (256) and the smallest
+beyond it; equal scores and repeated keys, whose ties go to the lower position; and the every-candidate
+selector's candidate counts around its warps' 32 rows and its block's 1024, with both signs of lambda2.
+Every admission is replayed through the oracle, margins included."""
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import kv_evict_oracle as O
+from paper_2609_30738_gb300 import synth
+from paper_2609_30738_gb300.workloads import WORKLOADS, scaled
+from tests import parity as PT
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2609_30738_gb300 import kv_evict
+    kv_evict.library()
+
+
+def _check(L, B, factor, lam2, seed, flat=False):
+    """Selection on given mu and sigma (flat: few distinct values, runs of equal keys)."""
+    from paper_2609_30738_gb300 import kv_evict as K
+    W, nl, hkv = 8, 2, 2
+    spec = scaled(WORKLOADS["mistral-1layer-L2048"], num_layers=nl, num_q_heads=4, num_kv_heads=hkv, window=W,
+                  budget=B, candidate_factor=factor, seq_lens=[L])
+    batch = synth.make_batch(spec, seed=seed, with_values=False)
+    rng = np.random.default_rng(seed)
+    mu = rng.random(nl * hkv * L).astype(np.float32) ** 4
+    sigma = rng.random(nl * hkv * L).astype(np.float32) ** 4
+    if flat:
+        mu, sigma = np.round(mu * 2) / 2 + np.float32(0.25), np.round(sigma * 2) / 2
+        batch["k"][:, :, 1::2] = batch["k"][:, :, 0:1]      # every other key is one and the same
+    mu, sigma = mu.astype(np.float32), sigma.astype(np.float32)
+    plan = K.Plan(spec, [L])
+    bufs = K.Buffers(plan)
+    bufs.mu.copy_(torch.from_numpy(mu))
+    bufs.sigma.copy_(torch.from_numpy(sigma))
+    bufs.ws.zero_()
+    l1, l2 = np.full(nl, 0.5, np.float32), np.full(nl, lam2, np.float32)
+    plan.select(bufs.mu, bufs.sigma, batch["k"].cuda(), l1, l2, bufs.indices, bufs.ws, bufs.order, bufs.margins)
+    assert plan.status(bufs.ws) == K.KVE_OK
+    order, indices = bufs.order.cpu().numpy(), bufs.indices.cpu().numpy()
+    margins = bufs.margins.cpu().numpy()
+    for u in range(nl * hkv):
+        keys = O.bf16_bits_to_f64(PT.to_bits(batch["k"][u // hkv, u % hkv]))
+        m64, s64 = mu[u * L:(u + 1) * L].astype(np.float64), sigma[u * L:(u + 1) * L].astype(np.float64)
+        PT.check_selection(order[u], indices[u], m64, s64, keys, L, W, B, 0.5, lam2, candidate_factor=factor,
+                           margins_gpu=margins[u])
+
+
+@pytest.mark.parametrize("lam2", [-0.5, 0.6, 0.0])
+@pytest.mark.parametrize("B,factor", [(127, 1), (64, 2), (43, 3), (51, 5), (64, 4), (257, 1)])
+def test_pool_edges(B, factor, lam2):
+    _check(1500, B, factor, lam2, seed=B)
+
+
+@pytest.mark.parametrize("lam2", [-0.5, 0.0])
+@pytest.mark.parametrize("L,B,factor", [(600, 32, 4), (600, 60, 4), (1500, 80, 4)])
+def test_pool_ties(L, B, factor, lam2):
+    _check(L, B, factor, lam2, seed=L + B, flat=True)
+
+
+@pytest.mark.parametrize("lam2", [-0.5, 0.6])
+@pytest.mark.parametrize("Lc", [513, 1023, 1025, 1056, 2081])
+def test_every_candidate_edges(Lc, lam2):
+    _check(Lc + 8, 24, 0, lam2, seed=Lc)
