@@ -14,14 +14,15 @@
 //     brings that candidate up to date (in parallel) and the search repeats; a
 //     candidate whose value is current when it is the best is the full greedy's
 //     choice (any candidate with an equal bound has a higher position).
-//     With lambda2 > 0 every candidate is brought up to date after each admission.
+//     With lambda2 > 0 every candidate is brought up to date after each admission, by
+//     warps that take 32 candidates at a time through the tensor cores.
 //     When margins are requested the runner-up is brought up to date the same way.
 //  3. write the admitted positions ascending (and in admission order, with margins).
 // Values live in shared memory (C <= 32768); s~, corr and the inverse key norms in
 // the workspace; the first 96 admitted keys are staged in shared memory, later ones
 // are read from K in global memory (L2). For lambda2 <= 0 a warp refreshes its lanes'
-// stale bests together on the tensor cores; for lambda2 > 0 a thread applies the
-// missing admissions in groups of eight per pass over the candidate's row.
+// stale bests together on the tensor cores; for lambda2 > 0 a warp forms the dots of 32
+// candidates with the key just admitted.
 #include "kve_internal.h"
 
 namespace kve {
@@ -31,7 +32,6 @@ constexpr int kAllThreads = 1024;
 constexpr int kAllWarps = kAllThreads / 32;
 constexpr int kAdmStage = 96;          // admitted keys staged in shared memory
 constexpr int kAdmStride = 17;         // uint4 per staged row (16 + 1 against bank conflicts)
-constexpr int kRefreshGroup = 8;       // missing admissions applied per pass over a candidate row
 
 __device__ __forceinline__ uint32_t ord_key_all(float f) {
   const uint32_t u = __float_as_uint(f + 0.0f);   // -0 -> +0
@@ -40,6 +40,35 @@ __device__ __forceinline__ uint32_t ord_key_all(float f) {
 
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
+
+__device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                         uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+      "{%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// The 32 candidate rows base .. base + 31 of a warp (rows past the last stand for it), 16 bytes
+// per load: lane (g, t) holds of row base + 8 r + g the 16-byte chunks 4 s + t (r, s = 0 .. 3), so
+// that a load instruction reads 64 contiguous bytes of each of 8 rows.
+__device__ __forceinline__ void load_rows(const uint16_t* kb, int64_t kst, int base, int C, uint4 (&x)[4][4]) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, tq = lane & 3;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const uint4* row = reinterpret_cast<const uint4*>(kb + static_cast<int64_t>(min(base + 8 * r + g, C - 1)) * kst);
+#pragma unroll
+    for (int s = 0; s < 4; ++s) x[r][s] = __ldg(row + 4 * s + tq);
+  }
+}
+
+// Of four values, one per row set r, the one of r = lane % 4: that lane's candidate is row
+// base + 8 (lane % 4) + lane / 4.
+__device__ __forceinline__ float own_row(const float (&y)[4]) {
+  const int tq = threadIdx.x & 3;
+  return tq < 2 ? (tq == 0 ? y[0] : y[1]) : (tq == 2 ? y[2] : y[3]);
+}
 
 struct AllSmall {
   uint32_t wkey[kAllWarps];
@@ -120,32 +149,46 @@ __global__ void __launch_bounds__(kAllThreads, 1) select_all_kernel(const __grid
   float smax = sh.wmax[0];
   for (int w = 1; w < kAllWarps; ++w) smax = fmaxf(smax, sh.wmax[w]);
   smax = fmaxf(smax, P.norm_eps);
-  for (int i = tid; i < C; i += kAllThreads) {
-    const float s = __fdiv_rn(st[i], smax);
-    st[i] = s;
-    v[i] = s;                     // corr = 0: s~ + lambda2 * 0
-    applied[i] = 0;
-    const uint4* ki = reinterpret_cast<const uint4*>(kb + static_cast<int64_t>(i) * kst);
-    float ss = 0.f;
-    for (int c = 0; c < kHeadDim / 8; ++c) {
-      const uint4 x = __ldg(ki + c);
-      const uint32_t w4[4] = {x.x, x.y, x.z, x.w};
+  // the owner of candidate i is the thread with own = i % kAllThreads: the lane whose row it is
+  // in load_rows; it keeps the best of its own candidates
+  const int own = warp * 32 + 8 * (lane & 3) + (lane >> 2);
+  for (int base = warp * 32; base < C; base += kAllThreads) {
+    uint4 x[4][4];
+    load_rows(kb, kst, base, C, x);
+    float ss[4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        ss = fmaf(bf16_lo(w4[e]), bf16_lo(w4[e]), ss);
-        ss = fmaf(bf16_hi(w4[e]), bf16_hi(w4[e]), ss);
+    for (int r = 0; r < 4; ++r) {
+      float e0 = 0.f, e1 = 0.f;
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        const uint32_t w4[4] = {x[r][s].x, x[r][s].y, x[r][s].z, x[r][s].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          e0 = fmaf(bf16_lo(w4[e]), bf16_lo(w4[e]), e0);
+          e1 = fmaf(bf16_hi(w4[e]), bf16_hi(w4[e]), e1);
+        }
       }
+      ss[r] = e0 + e1;
+      ss[r] += __shfl_xor_sync(0xffffffffu, ss[r], 1);
+      ss[r] += __shfl_xor_sync(0xffffffffu, ss[r], 2);
     }
-    cinv[i] = make_float2(0.f, ss > 0.f ? __fdiv_rn(1.0f, sqrtf(ss)) : 0.f);
+    const float n2 = own_row(ss);
+    const int i = base + 8 * (lane & 3) + (lane >> 2);
+    if (i < C) {
+      const float s = __fdiv_rn(st[i], smax);
+      st[i] = s;
+      v[i] = s;                     // corr = 0: s~ + lambda2 * 0
+      applied[i] = 0;
+      cinv[i] = make_float2(0.f, n2 > 0.f ? __fdiv_rn(1.0f, sqrtf(n2)) : 0.f);
+    }
   }
   __syncthreads();
 
-  // the owner of candidate i is thread i % kAllThreads; it keeps the best of its own
   uint32_t my_key = 0, my_idx = 0xFFFFFFFFu;
   auto rescan = [&]() {
     my_key = 0;
     my_idx = 0xFFFFFFFFu;
-    for (int i = tid; i < C; i += kAllThreads) {
+    for (int i = own; i < C; i += kAllThreads) {
       const float x = v[i];
       if (x == -INFINITY) continue;   // admitted
       const uint32_t k = ord_key_all(x);
@@ -157,57 +200,60 @@ __global__ void __launch_bounds__(kAllThreads, 1) select_all_kernel(const __grid
   };
   rescan();
 
-  // candidate i brought up to date with admissions applied[i] .. t-1 by its owner,
-  // kRefreshGroup admissions per pass over the candidate's row (each dot keeps the
-  // element order of a plain loop); staged admitted keys come from shared memory
-  auto refresh = [&](int i, int t) {
-    const uint4* ki = reinterpret_cast<const uint4*>(kb + static_cast<int64_t>(i) * kst);
-    const float2 ci = cinv[i];
-    const float inv_i = ci.y;
-    float cmax = ci.x;
-    // admitted key a, chunk c: staged in shared memory or read from K
-    auto adm_chunk = [&](int a, int c) -> uint4 {
-      return a < kAdmStage ? admk[a * kAdmStride + c]
-                           : __ldg(reinterpret_cast<const uint4*>(kb + static_cast<int64_t>(adm[a]) * kst) + c);
-    };
-    int a0 = applied[i];
-    for (; a0 + kRefreshGroup <= t; a0 += kRefreshGroup) {
-      float dot[kRefreshGroup];
+  // lambda2 > 0: every candidate brought up to date with the admission of key a, and the owners'
+  // new bests. The dots of 32 candidates with that key are 16 mma.m16n8k16 per warp: candidate
+  // rows as A fragments straight from the 16-byte loads (a dot does not depend on the order of
+  // its elements, so chunk 4 s + t of a row and of the admitted key stand for the k-steps' lane t),
+  // the key in every column of B. Bound by the keys' read from L2 (1 MB per admission at 4096
+  // candidates): 6 layers of 4096 tokens, two of them with lambda2 > 0, took 2.88 ms with a
+  // thread per candidate on the FMA pipe.
+  auto refresh_all = [&](int a) {
+    const uint4* src = a < kAdmStage ? admk + a * kAdmStride
+                                     : reinterpret_cast<const uint4*>(kb + static_cast<int64_t>(adm[a]) * kst);
+    uint4 y[4];
 #pragma unroll
-      for (int q = 0; q < kRefreshGroup; ++q) dot[q] = 0.f;
-      for (int c = 0; c < kHeadDim / 8; ++c) {
-        const uint4 x = __ldg(ki + c);
-        const uint32_t xa[4] = {x.x, x.y, x.z, x.w};
+    for (int s = 0; s < 4; ++s) y[s] = src[4 * s + (lane & 3)];
+    const float inv_a = adm_inv[a];
+    my_key = 0;
+    my_idx = 0xFFFFFFFFu;
+    for (int base = warp * 32; base < C; base += kAllThreads) {
+      uint4 x[4][4];
+      load_rows(kb, kst, base, C, x);
+      const int i = base + 8 * (lane & 3) + (lane >> 2);
+      const float2 ci = i < C ? cinv[i] : make_float2(0.f, 0.f);
+      const float si = i < C ? st[i] : 0.f;
+      float d[2][2][4];   // [m-tile][chain]
 #pragma unroll
-        for (int q = 0; q < kRefreshGroup; ++q) {
-          const uint4 y = adm_chunk(a0 + q, c);
-          const uint32_t ya[4] = {y.x, y.y, y.z, y.w};
+      for (int m = 0; m < 2; ++m)
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            dot[q] = fmaf(bf16_lo(xa[e]), bf16_lo(ya[e]), dot[q]);
-            dot[q] = fmaf(bf16_hi(xa[e]), bf16_hi(ya[e]), dot[q]);
-          }
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) d[m][c][e] = 0.f;
+#pragma unroll
+      for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+          const uint4 r0 = x[2 * m][s], r1 = x[2 * m + 1][s];
+          mma_bf16(d[m][0], r0.x, r1.x, r0.y, r1.y, y[s].x, y[s].y);
+          mma_bf16(d[m][1], r0.z, r1.z, r0.w, r1.w, y[s].z, y[s].w);
+        }
+      // element 0 is row g of the m-tile, element 2 row g + 8; every column holds the same dot
+      const float dots[4] = {d[0][0][0] + d[0][1][0], d[0][0][2] + d[0][1][2],
+                             d[1][0][0] + d[1][1][0], d[1][0][2] + d[1][1][2]};
+      const float dot = own_row(dots);
+      if (i < C && v[i] != -INFINITY) {   // not admitted
+        const float cm = fmaxf(ci.x, dot * ci.y * inv_a);
+        const float val = fmaf(lambda2, cm, si);
+        cinv[i].x = cm;
+        v[i] = val;
+        applied[i] = static_cast<uint16_t>(a + 1);
+        const uint32_t k = ord_key_all(val);
+        if (k > my_key || my_idx == 0xFFFFFFFFu) {
+          my_key = k;
+          my_idx = static_cast<uint32_t>(i);
         }
       }
-#pragma unroll
-      for (int q = 0; q < kRefreshGroup; ++q) cmax = fmaxf(cmax, dot[q] * inv_i * adm_inv[a0 + q]);
     }
-    for (; a0 < t; ++a0) {
-      float dot = 0.f;
-      for (int c = 0; c < kHeadDim / 8; ++c) {
-        const uint4 x = __ldg(ki + c), y = adm_chunk(a0, c);
-        const uint32_t xa[4] = {x.x, x.y, x.z, x.w}, ya[4] = {y.x, y.y, y.z, y.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          dot = fmaf(bf16_lo(xa[e]), bf16_lo(ya[e]), dot);
-          dot = fmaf(bf16_hi(xa[e]), bf16_hi(ya[e]), dot);
-        }
-      }
-      cmax = fmaxf(cmax, dot * inv_i * adm_inv[a0]);
-    }
-    cinv[i] = make_float2(cmax, inv_i);
-    v[i] = fmaf(lambda2, cmax, st[i]);
-    applied[i] = static_cast<uint16_t>(t);
   };
   // every owner whose best is stale brings it up to date, then takes its new best.
   // A warp refreshes its lanes' stale bests together on the tensor cores: lane r's
@@ -273,12 +319,7 @@ __global__ void __launch_bounds__(kAllThreads, 1) select_all_kernel(const __grid
             const uint32_t b1 = bv[n] ? rb[n][8 * s8 + tq + 4] : 0u;
 #pragma unroll
             for (int m = 0; m < 2; ++m) {
-              float* dd = d[m][n];
-              asm volatile(
-                  "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
-                  "{%8,%9}, {%0,%1,%2,%3};"
-                  : "+f"(dd[0]), "+f"(dd[1]), "+f"(dd[2]), "+f"(dd[3])
-                  : "r"(af[m][0]), "r"(af[m][1]), "r"(af[m][2]), "r"(af[m][3]), "r"(b0), "r"(b1));
+              mma_bf16(d[m][n], af[m][0], af[m][1], af[m][2], af[m][3], b0, b1);
             }
           }
         }
@@ -348,7 +389,7 @@ __global__ void __launch_bounds__(kAllThreads, 1) select_all_kernel(const __grid
       admk[t * kAdmStride + tid] =
           __ldg(reinterpret_cast<const uint4*>(kb + static_cast<int64_t>(bi) * kst) + tid);
     __syncthreads();
-    if (tid == (bi % kAllThreads)) rescan();
+    if (own == (bi % kAllThreads)) rescan();
     if (margins) {
       // the runner-up, brought up to date against admissions 0 .. t-1
       for (;;) {
@@ -369,13 +410,8 @@ __global__ void __launch_bounds__(kAllThreads, 1) select_all_kernel(const __grid
     if (tid == 0) adm_inv[t] = cinv[bi].y;   // inverse norm of the admitted key
     __syncthreads();
     ++t;
-    if (!lazy && t < nsel) {
-      // lambda2 > 0: values grow with corr, so every candidate is brought up to date
-      for (int i = tid; i < C; i += kAllThreads)
-        if (v[i] != -INFINITY) refresh(i, t);
-      __syncthreads();
-      rescan();
-    }
+    // lambda2 > 0: values grow with corr, so every candidate is brought up to date (by its owner)
+    if (!lazy && t < nsel) refresh_all(t - 1);
   }
 
   // 3. admitted positions ascending, then -1: entry a of the admission order goes to
