@@ -43,7 +43,8 @@ constexpr int kTieCap = 2048;           // cut ties gathered in shared memory
 
 __device__ __forceinline__ uint32_t ord_key(float f) {
   const uint32_t u = __float_as_uint(f + 0.0f);   // -0 -> +0
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+  // negative: ~u, otherwise u with the sign bit set
+  return u ^ (static_cast<uint32_t>(static_cast<int32_t>(u) >> 31) | 0x80000000u);
 }
 
 // max of three floats in one instruction
@@ -82,7 +83,7 @@ constexpr uint64_t kGramWaitNs = 2000000000ull;
 template <int NT>
 struct SelSmall {
   uint64_t gram_bar[3];          // G01, G11, G00 formed
-  uint4 win[2][2];               // per warp of the greedy: best keys and tie keys, by step parity
+  uint4 win[2][2];               // per warp of the greedy: (best key, tie key), by step parity
   uint32_t wsec[2][4];           // and second keys
   uint32_t tmem;
   volatile int abort;            // never set: the waits here have no other party
@@ -262,22 +263,60 @@ __device__ __forceinline__ bool gram_form(SelSmall<NT>& sh, uint8_t* keys, int n
   return true;
 }
 
+// The squared norm of slot threadIdx.x from the diagonal of G00 or G11. Whole warps.
+__device__ __forceinline__ float gram_diagonal(uint32_t tmem) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t quad = static_cast<uint32_t>(warp & 3) * 32u;
+  float v[32];
+  tmem_ld32(tmem + (quad << 16) + 128u * (warp >> 2) + quad, v);
+  tmem_wait_ld(v);
+  float d = 0.f;
+#pragma unroll
+  for (int j = 0; j < 32; ++j) d = j == lane ? v[j] : d;
+  return d;
+}
+
+// 1 / sqrt(x) as the sum of two floats, for x in [2^-64, 2^120].
+__device__ __forceinline__ float2 inv_sqrt2(float x) {
+  const float y = inv_sqrt(x);
+  const float p = x * y;
+  const float r = fmaf(-p, y, 1.0f) - fmaf(x, y, -p) * y;   // 1 - x y^2
+  return make_float2(y, 0.5f * y * r);
+}
+
+// dot * a * b with a and b in two floats each, rounded once.
+__device__ __forceinline__ float cosine(float dot, float2 a, float2 b) {
+  const float p = a.x * b.x;
+  const float e = fmaf(a.x, b.x, -p) + fmaf(a.x, b.y, a.y * b.x);
+  return fmaf(dot, p, dot * e);
+}
+
 // The greedy over a pool of up to 256 slots whose dot products stand (gram_form): warps 0 .. 3,
 // thread i owns slots i and 128 + i. A step is a chain of latencies -- two warp reductions, one
 // barrier of the four warps, the fold of their results -- after which the admitted slot's dots
-// are one TMEM column and one shared-memory row or column: 0.29 us, against 0.53 us with the dots
-// of every admission formed when it is known (16 mma.sync per warp, whose 8 columns all held the
-// same key). 64 admissions: 18.7 us per unit and 2.5 us for the products, against 33.8; a launch
-// of 256 units of 8192 tokens 44.6 us against 58.5, of 32768 tokens 72.1 against 82. st[], inv: normalised base score and inverse norm of the thread's slots (inactive
-// slots: `active` false); tie: position << 9 | slot or the slot.
+// are one TMEM column and one shared-memory row or column: under 0.3 us, against 0.53 us with the
+// dots of every admission formed when it is known (16 mma.sync per warp, whose 8 columns all held
+// the same key). Positions, slots and the order are decoded from the tie keys after the loop. A
+// launch of 256 units and 64 admissions takes 42 us instead of 58 at 8192 tokens, 66 instead of
+// 82 at 32768.
+// The products are summed along one chain of eight MMAs, which truncates. The norms come from the
+// diagonal, the same chain, so that this bias cancels in the cosine, and the inverse norms are
+// kept in two floats, so that the cosine is rounded once. Error of the margins against 64 bits
+// (same mu and sigma, 3000 tokens): 1.20e-8 rms at lambda2 = -0.5 and 4.53e-8 at 0.6, against
+// 1.50e-8 and 5.39e-8 with four chains of two MMAs and norms of two fp32 chains; with those norms
+// and the one chain it was 1.71e-8 and 6.37e-8.
+// st: normalised base score; inv: inverse norm (of inactive slots: `active` false); tie: position
+// << 9 | slot, or the slot. ties[t] receives admission t's tie key.
 struct GreedySlot {
-  float st, inv, corr;
+  float st, corr;
+  float2 inv;
   uint32_t tie;
   bool active;
 };
-template <int NT, class Admit>
-__device__ __forceinline__ void gram_greedy(SelSmall<NT>& sh, const float* g01, const float* inv, GreedySlot (&s)[2],
-                                            float lambda2, int nsel, bool packed, bool want_second, Admit admit) {
+template <int NT, class Margin>
+__device__ __forceinline__ void gram_greedy(SelSmall<NT>& sh, const float* g01, const float2* inv, GreedySlot (&s)[2],
+                                            float lambda2, int nsel, bool packed, uint32_t* ties,
+                                            bool want_second, Margin margin) {
   const int i = threadIdx.x, warp = i >> 5, lane = i & 31;
   const uint32_t tcol = sh.tmem + (static_cast<uint32_t>(warp * 32) << 16);
   for (int t = 0; t < nsel; ++t) {
@@ -294,19 +333,18 @@ __device__ __forceinline__ void gram_greedy(SelSmall<NT>& sh, const float* g01, 
     uint32_t wtie = tie;   // of the only holder, or the smallest
     if (holders & (holders - 1u)) wtie = __reduce_min_sync(0xffffffffu, key == wmax ? tie : 0xFFFFFFFFu);
     const bool mine = key == wmax && tie == wtie;
-    if (mine) {
-      reinterpret_cast<uint32_t*>(&sh.win[t & 1][0])[warp] = key;
-      reinterpret_cast<uint32_t*>(&sh.win[t & 1][1])[warp] = tie;
-    }
+    if (mine) reinterpret_cast<uint2*>(&sh.win[t & 1][0])[warp] = make_uint2(key, tie);
     if (want_second) {
       const uint32_t wsec = __reduce_max_sync(0xffffffffu, mine ? (second ? k[0] : k[1]) : key);
       if (lane == 0) sh.wsec[t & 1][warp] = wsec;
     }
     named_bar_sync(1, 128);
-    const uint4 wk = sh.win[t & 1][0], wt = sh.win[t & 1][1];
+    const uint4 w01 = sh.win[t & 1][0], w23 = sh.win[t & 1][1];
     // the largest key, then the smallest tie key
-    const bool b01 = wk.y > wk.x || (wk.y == wk.x && wt.y < wt.x), b23 = wk.w > wk.z || (wk.w == wk.z && wt.w < wt.z);
-    const uint32_t ka = b01 ? wk.y : wk.x, ta = b01 ? wt.y : wt.x, kb = b23 ? wk.w : wk.z, tb = b23 ? wt.w : wt.z;
+    const bool b01 = w01.z > w01.x || (w01.z == w01.x && w01.w < w01.y);
+    const bool b23 = w23.z > w23.x || (w23.z == w23.x && w23.w < w23.y);
+    const uint32_t ka = b01 ? w01.z : w01.x, ta = b01 ? w01.w : w01.y;
+    const uint32_t kb = b23 ? w23.z : w23.x, tb = b23 ? w23.w : w23.y;
     const bool b = kb > ka || (kb == ka && tb < ta);
     const uint32_t best = b ? kb : ka, btie = b ? tb : ta;
     const int js = static_cast<int>((packed ? (btie & 511u) : btie) & (kGramCols - 1u));
@@ -314,25 +352,23 @@ __device__ __forceinline__ void gram_greedy(SelSmall<NT>& sh, const float* g01, 
     // the dots with slot js: within its half in TMEM (column js), across in g01
     const float tm = tmem_ld1(tcol + static_cast<uint32_t>(js));
     const float of = js < 128 ? g01[jj * kGramPitch + i] : g01[i * kGramPitch + jj];
-    const float inv_j = inv[js];
-    if (i == 0) {
+    const float2 inv_j = inv[js];
+    if (i == 0) ties[t] = btie;
+    if (want_second && i == 0) {
+      // runner-up: the other warps' best and the winning warp's second
+      const int w = b ? (b23 ? 3 : 2) : (b01 ? 1 : 0);
+      const uint32_t all[4] = {w01.x, w01.z, w23.x, w23.z};
       uint32_t sec = 0u;
-      if (want_second) {
-        // runner-up: the other warps' best and the winning warp's second
-        const int w = b ? (b23 ? 3 : 2) : (b01 ? 1 : 0);
-        const uint32_t all[4] = {wk.x, wk.y, wk.z, wk.w};
 #pragma unroll
-        for (int e = 0; e < 4; ++e) sec = max(sec, e == w ? sh.wsec[t & 1][e] : all[e]);
-      }
-      admit(t, js, btie, best, sec);
+      for (int e = 0; e < 4; ++e) sec = max(sec, e == w ? sh.wsec[t & 1][e] : all[e]);
+      margin(t, best, sec);
     }
-    if (i == jj) {
-      if (js < 128) s[0].active = false; else s[1].active = false;
-    }
+    s[0].active = s[0].active && i != js;
+    s[1].active = s[1].active && i + 128 != js;
     tmem_wait_ld();
     const float d0 = js < 128 ? tm : of, d1 = js < 128 ? of : tm;
-    s[0].corr = fmaxf(s[0].corr, d0 * s[0].inv * inv_j);
-    s[1].corr = fmaxf(s[1].corr, d1 * s[1].inv * inv_j);
+    s[0].corr = fmaxf(s[0].corr, cosine(d0, s[0].inv, inv_j));
+    s[1].corr = fmaxf(s[1].corr, cosine(d1, s[1].inv, inv_j));
   }
 }
 
@@ -695,6 +731,18 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
   __syncthreads();
   const uint32_t ncand = sh.ncand;
   const bool staged = ncand <= kCandCap<NT>();
+  // The unit reports no selection.
+  auto no_selection = [&](uint32_t why) {
+    if (tid == 0 && P.err) atomicOr(P.err, why);
+    int32_t* out = P.indices + out_off + u.unit * B;
+    for (int r = tid; r < B; r += NT) out[r] = -1;
+    if (P.order)
+      for (int r = tid; r < B; r += NT) P.order[out_off + u.unit * B + r] = -1;
+    if (P.margins)
+      for (int r = tid; r < B; r += NT) P.margins[out_off + u.unit * B + r] = 0.f;
+    if (P.k_out) write_compact_cache<NT>(P, u, Lc, nsel, 0, nullptr, nullptr, nullptr);
+  };
+
   digit_pass(1, 0xFFFu << 20, staged, ncand);
   digit_pass(2, 0xFFFFFFu << 8, staged, ncand);
   const uint32_t T = sh.prefix;
@@ -756,16 +804,6 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
   // exactly C positions (the pool writes above are bounded by the pool's size all the
   // same). Should that ever fail, the pool would hold unwritten slots: the unit is then
   // reported through the error word and gets no selection.
-  auto no_selection = [&](uint32_t why) {
-    if (tid == 0 && P.err) atomicOr(P.err, why);
-    int32_t* out = P.indices + out_off + u.unit * B;
-    for (int r = tid; r < B; r += NT) out[r] = -1;
-    if (P.order)
-      for (int r = tid; r < B; r += NT) P.order[out_off + u.unit * B + r] = -1;
-    if (P.margins)
-      for (int r = tid; r < B; r += NT) P.margins[out_off + u.unit * B + r] = 0.f;
-    if (P.k_out) write_compact_cache<NT>(P, u, Lc, nsel, 0, nullptr, nullptr, nullptr);
-  };
   if (n_above + needT != static_cast<uint32_t>(C) || needT > n_eq || needT == 0u) {
     no_selection(kErrCheck);
     if constexpr (kGram) {
@@ -857,7 +895,7 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
   // and their slots when the compact cache is written here
   int32_t* adm = packed ? spos : cpos;
   int32_t* adm_slot = reinterpret_cast<int32_t*>(packed ? skey : ckey);
-  // the inverse norm of a staged row: its squares summed in two chains
+  // the inverse norm of a key row: its squares summed in two chains
   auto row_inv_norm = [](auto chunk) {
     float ss0 = 0.f, ss1 = 0.f;
 #pragma unroll 4
@@ -882,10 +920,19 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
     // 5. greedy admissions on the pool's dot products
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the keys are read by the MMAs
     __syncthreads();
-    // a slot's inverse norm from its own staged row
-    if (tid < C) inv[tid] = row_inv_norm([&](int c) { return *reinterpret_cast<const uint4*>(gram_chunk(big, tid, c)); });
-    __syncthreads();
     const bool formed = gram_form<NT>(sh, big, C > 128 ? 2 : 1);
+    float2* inv2 = reinterpret_cast<float2*>(hist0);   // (the first digit's histogram is dead)
+    if (formed && tid < ((C + 31) & ~31)) {            // whole warps
+      const float ss = gram_diagonal(sh.tmem);
+      if (ss >= 0x1p-64f && ss <= 0x1p120f)
+        inv2[tid] = inv_sqrt2(ss);
+      else if (tid < C) {
+        // sums that tensor cores may flush or cut off: from the key itself
+        const uint4* src = reinterpret_cast<const uint4*>(P.k + u.k_off + ppos[tid] * P.g.k_st);
+        inv2[tid] = make_float2(row_inv_norm([&](int c) { return __ldg(src + c); }), 0.f);
+      }
+    }
+    __syncthreads();
     if (formed && warp < 4) {
       GreedySlot s[2];
 #pragma unroll
@@ -893,20 +940,26 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
         const int slot = tid + 128 * e;
         s[e].active = slot < C;
         s[e].st = s[e].active ? __fdiv_rn(unord_key(pkey[slot]), smax) : 0.f;
-        s[e].inv = s[e].active ? inv[slot] : 0.f;
+        s[e].inv = s[e].active ? inv2[slot] : make_float2(0.f, 0.f);
         s[e].corr = 0.f;
         s[e].tie = s[e].active ? tie_key(slot) : 0xFFFFFFFFu;
       }
-      gram_greedy<NT>(sh, reinterpret_cast<const float*>(big), inv, s, lambda2, nsel, packed, margins != nullptr,
-                      [&](int t, int js, uint32_t btie, uint32_t best, uint32_t sec) {
-                        const int pos = packed ? static_cast<int>(btie >> 9) : ppos[js];
-                        adm[t] = pos;
-                        adm_slot[t] = js;
-                        if (order) order[t] = pos;
-                        if (margins) margins[t] = sec ? unord_key(best) - unord_key(sec) : INFINITY;
+      gram_greedy<NT>(sh, reinterpret_cast<const float*>(big), inv2, s, lambda2, nsel, packed,
+                      reinterpret_cast<uint32_t*>(adm_slot), margins != nullptr,
+                      [&](int t, uint32_t best, uint32_t sec) {
+                        margins[t] = sec ? unord_key(best) - unord_key(sec) : INFINITY;
                       });
     }
     tc_fence_before();
+    __syncthreads();
+    for (int t = tid; t < nsel; t += NT) {
+      const uint32_t tie = static_cast<uint32_t>(adm_slot[t]);
+      const int js = static_cast<int>(packed ? (tie & 511u) : tie);
+      const int pos = packed ? static_cast<int>(tie >> 9) : ppos[js];
+      adm[t] = pos;
+      adm_slot[t] = js;
+      if (order) order[t] = pos;
+    }
     __syncthreads();
     if (warp == 0) {
       tc_fence_after();

@@ -1,7 +1,8 @@
 """Pool sizes at the edges of the selector's greedy: one half of 128 slots and two, a slot short of a
 half and one past it, the largest pool whose dot products stand before the greedy (256) and the smallest
 beyond it; equal scores and repeated keys, whose ties go to the lower position; and the every-candidate
-selector's candidate counts around its warps' 32 rows and its block's 1024, with both signs of lambda2.
+selector's candidate counts around its warps' 32 rows and its block's 1024, with both signs of lambda2;
+very small, very large and zero keys.
 Every admission is replayed through the oracle, margins included."""
 
 import numpy as np
@@ -25,8 +26,8 @@ def _lib():
     kv_evict.library()
 
 
-def _check(L, B, factor, lam2, seed, flat=False):
-    """Selection on given mu and sigma (flat: few distinct values, runs of equal keys)."""
+def _check(L, B, factor, lam2, seed, flat=False, scale=1.0):
+    """Selection on given mu and sigma (flat: few distinct values, runs of equal keys; scale: of the keys)."""
     from paper_2609_30738_gb300 import kv_evict as K
     W, nl, hkv = 8, 2, 2
     spec = scaled(WORKLOADS["mistral-1layer-L2048"], num_layers=nl, num_q_heads=4, num_kv_heads=hkv, window=W,
@@ -39,6 +40,9 @@ def _check(L, B, factor, lam2, seed, flat=False):
         mu, sigma = np.round(mu * 2) / 2 + np.float32(0.25), np.round(sigma * 2) / 2
         batch["k"][:, :, 1::2] = batch["k"][:, :, 0:1]      # every other key is one and the same
     mu, sigma = mu.astype(np.float32), sigma.astype(np.float32)
+    if scale != 1.0:
+        batch["k"] *= scale
+        batch["k"][:, :, 5::7] = 0
     plan = K.Plan(spec, [L])
     bufs = K.Buffers(plan)
     bufs.mu.copy_(torch.from_numpy(mu))
@@ -72,3 +76,10 @@ def test_pool_ties(L, B, factor, lam2):
 @pytest.mark.parametrize("Lc", [513, 1023, 1025, 1056, 2081])
 def test_every_candidate_edges(Lc, lam2):
     _check(Lc + 8, 24, 0, lam2, seed=Lc)
+
+
+@pytest.mark.parametrize("B", [30, 60])
+@pytest.mark.parametrize("scale", [2.0 ** -40, 2.0 ** -31, 2.0 ** 58])
+def test_pool_key_scales(scale, B):
+    """Squared norms below, around and above the range in which they are read from the dots; zero keys."""
+    _check(700, B, 4, -0.5, seed=B, scale=scale)
