@@ -10,10 +10,10 @@
 //     corr_i = max over admitted j of cos(k_i, k_j) (clamped at 0 by starting at 0).
 //     With lambda2 <= 0 a value can only fall as the admitted set grows, so a value
 //     computed against fewer admitted keys is an upper bound: each step takes the
-//     best value; if it is stale, every thread whose own best candidate is stale
-//     brings that candidate up to date (in parallel) and the search repeats; a
-//     candidate whose value is current when it is the best is the full greedy's
-//     choice (any candidate with an equal bound has a higher position).
+//     best value; if it is stale, the threads whose own best candidate is stale and
+//     could still be the admission bring it up to date (in parallel) and the search
+//     repeats; a candidate whose value is current when it is the best is the full
+//     greedy's choice (any candidate with an equal bound has a higher position).
 //     With lambda2 > 0 every candidate is brought up to date after each admission, by
 //     warps that take 32 candidates at a time through the tensor cores.
 //     When margins are requested the runner-up is brought up to date the same way.
@@ -28,7 +28,9 @@
 namespace kve {
 namespace {
 
-constexpr int kAllThreads = 1024;
+// 128 registers a thread: with 1024 threads of 64 the selector spilled, and shared memory leaves the
+// spills hardly any L1 (lambda2 > 0 over 4064 candidates: 1.28 ms against 0.82).
+constexpr int kAllThreads = 512;
 constexpr int kAllWarps = kAllThreads / 32;
 constexpr int kAdmStage = 96;          // admitted keys staged in shared memory
 constexpr int kAdmStride = 17;         // uint4 per staged row (16 + 1 against bank conflicts)
@@ -36,6 +38,10 @@ constexpr int kAdmStride = 17;         // uint4 per staged row (16 + 1 against b
 __device__ __forceinline__ uint32_t ord_key_all(float f) {
   const uint32_t u = __float_as_uint(f + 0.0f);   // -0 -> +0
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+
+__device__ __forceinline__ float unord_key_all(uint32_t k) {
+  return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
 }
 
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
@@ -71,29 +77,40 @@ __device__ __forceinline__ float own_row(const float (&y)[4]) {
 }
 
 struct AllSmall {
-  uint32_t wkey[kAllWarps];
+  uint32_t wkey[kAllWarps];    // per warp: its owners' best, and the best that is current
   uint32_t widx[kAllWarps];
+  uint32_t wcur[kAllWarps];
   float wmax[kAllWarps];
-  uint32_t best_key, best_idx;
+  uint32_t best_key, best_idx, cur_key;
+  bool stale;                  // the block's best is a bound, not its current value
 };
 
-// Block argmax of the owners' bests: the largest key, ties to the lowest index.
-__device__ __forceinline__ void block_best(uint32_t key, uint32_t idx, AllSmall& sh) {
+// Block argmax of the owners' bests: the largest key, ties to the lowest index; and the largest
+// of the owners' best current keys, `cur` (0: none has one).
+__device__ __forceinline__ void block_best(uint32_t key, uint32_t idx, uint32_t cur, const uint16_t* applied, int t,
+                                           AllSmall& sh) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t wk = __reduce_max_sync(0xffffffffu, key);
   const uint32_t wi = __reduce_min_sync(0xffffffffu, key == wk ? idx : 0xFFFFFFFFu);
+  const uint32_t wc = __reduce_max_sync(0xffffffffu, cur);
   if (lane == 0) {
     sh.wkey[warp] = wk;
     sh.widx[warp] = wi;
+    sh.wcur[warp] = wc;
   }
   __syncthreads();
   if (warp == 0) {
-    const uint32_t k = sh.wkey[lane], i = sh.widx[lane];
+    const bool hold = lane < kAllWarps;
+    const uint32_t k = hold ? sh.wkey[lane] : 0u, i = hold ? sh.widx[lane] : 0xFFFFFFFFu;
     const uint32_t bk = __reduce_max_sync(0xffffffffu, k);
     const uint32_t bi = __reduce_min_sync(0xffffffffu, k == bk ? i : 0xFFFFFFFFu);
+    const uint32_t bc = __reduce_max_sync(0xffffffffu, hold ? sh.wcur[lane] : 0u);
     if (lane == 0) {
       sh.best_key = bk;
       sh.best_idx = bi;
+      sh.cur_key = bc;
+      // read here, between the barriers: the owner may bring it up to date after the second
+      sh.stale = bi != 0xFFFFFFFFu && applied[bi] < t;
     }
   }
   __syncthreads();
@@ -185,28 +202,31 @@ __global__ void __launch_bounds__(kAllThreads, 1) select_all_kernel(const __grid
   __syncthreads();
 
   uint32_t my_key = 0, my_idx = 0xFFFFFFFFu;
-  auto rescan = [&]() {
+  uint32_t my_cur = 0;   // and the best key of those that hold t applied admissions
+  auto rescan = [&](int t) {
+    my_cur = 0;
     my_key = 0;
     my_idx = 0xFFFFFFFFu;
     for (int i = own; i < C; i += kAllThreads) {
       const float x = v[i];
       if (x == -INFINITY) continue;   // admitted
       const uint32_t k = ord_key_all(x);
+      if (applied[i] >= t) my_cur = max(my_cur, k);
       if (k > my_key || my_idx == 0xFFFFFFFFu) {
         my_key = k;
         my_idx = static_cast<uint32_t>(i);
       }
     }
   };
-  rescan();
+  rescan(0);
 
   // lambda2 > 0: every candidate brought up to date with the admission of key a, and the owners'
   // new bests. The dots of 32 candidates with that key are 16 mma.m16n8k16 per warp: candidate
   // rows as A fragments straight from the 16-byte loads (a dot does not depend on the order of
   // its elements, so chunk 4 s + t of a row and of the admitted key stand for the k-steps' lane t),
-  // the key in every column of B. Bound by the keys' read from L2 (1 MB per admission at 4096
-  // candidates): 6 layers of 4096 tokens, two of them with lambda2 > 0, took 2.88 ms with a
-  // thread per candidate on the FMA pipe.
+  // the key in every column of B. Bound by the keys' read from L2 (1 MB per admission at 4064
+  // candidates): 64 admissions over 4064 candidates take 0.82 ms, against 2.88 with a thread per
+  // candidate on the FMA pipe.
   auto refresh_all = [&](int a) {
     const uint4* src = a < kAdmStage ? admk + a * kAdmStride
                                      : reinterpret_cast<const uint4*>(kb + static_cast<int64_t>(adm[a]) * kst);
@@ -255,163 +275,137 @@ __global__ void __launch_bounds__(kAllThreads, 1) select_all_kernel(const __grid
       }
     }
   };
-  // every owner whose best is stale brings it up to date, then takes its new best.
-  // A warp refreshes its lanes' stale bests together on the tensor cores: lane r's
-  // candidate row is row r of the A operand of mma.m16n8k16 (two m-tiles), the
-  // admitted keys a_lo .. t-1 form the B operand, 16 per pass (two n-tiles), where
-  // a_lo is the smallest count applied among the warp's stale bests; a dot against
-  // an admission already applied leaves the running maximum unchanged.
-  const uint32_t* kw32 = reinterpret_cast<const uint32_t*>(kb);          // row i at kw32 + i * kst / 2
-  const int64_t kst32 = kst / 2;
-  const uint32_t* admw = reinterpret_cast<const uint32_t*>(admk);        // 4 * kAdmStride words per row
-  auto refresh_stale_bests = [&](int t) {
-    const bool stale = my_idx != 0xFFFFFFFFu && applied[my_idx] < t;
-    if (__any_sync(0xffffffffu, stale)) {
+  // lambda2 <= 0: after a search whose best is stale, the owners whose stale best could still be
+  // the admission bring it up to date and take their new best: those at or above the best current
+  // value, or, while there is no current value, the best of each warp. A round is a chain of
+  // latencies, so that few rows a round pay although they make more rounds. 64 admissions at
+  // lambda2 = -0.9: over 4064 candidates 0.61 ms, over 19968 2.01 ms; with every owner's stale best
+  // brought up to date in each round (512 to 1024 rows, 34 to 50 % fewer rounds) 1.73 and 3.27 ms.
+  // A warp does this for its lanes together on the tensor cores: lane r's candidate row is row r
+  // of the A operand of mma.m16n8k16 (two m-tiles, each skipped when no lane of it takes part),
+  // the admitted keys a_lo .. t-1 form the B operand, 8 per pass, where a_lo is the smallest count
+  // applied among these bests; a dot with an admission already applied leaves the running maximum
+  // unchanged. The rows are loaded 16 bytes at a time, as in load_rows.
+  auto refresh_bests = [&](int t) {
+    const uint32_t cur = sh.cur_key;
+    const bool want = my_idx != 0xFFFFFFFFu && applied[my_idx] < t &&
+                      (cur != 0u ? my_key >= cur : my_idx == sh.widx[warp]);
+    const uint32_t wants = __ballot_sync(0xffffffffu, want);
+    if (wants) {
       const int a_lo = static_cast<int>(__reduce_min_sync(
-          0xffffffffu, stale ? static_cast<uint32_t>(applied[my_idx]) : static_cast<uint32_t>(t)));
-      const int row = stale ? static_cast<int>(my_idx) : 0;      // row 0: a valid stand-in
-      const float2 ci = stale ? cinv[my_idx] : make_float2(0.f, 0.f);
+          0xffffffffu, want ? static_cast<uint32_t>(applied[my_idx]) : static_cast<uint32_t>(t)));
+      const float2 ci = want ? cinv[my_idx] : make_float2(0.f, 0.f);
+      const int any = __shfl_sync(0xffffffffu, static_cast<int>(my_idx), __ffs(wants) - 1);
+      const int row = want ? static_cast<int>(my_idx) : any;   // a valid stand-in
       float cm = ci.x;
       const int g = lane >> 2, tq = lane & 3;
-      // rows g and g + 8 of m-tiles 0 and 1 belong to lanes 16m + 8hh + g
-      const uint32_t* ra[2][2];
-      float ir[2][2];
+#pragma unroll 1
+      for (int m = 0; m < 2; ++m) {
+        if (((wants >> (16 * m)) & 0xFFFFu) == 0u) continue;
+        // rows g and g + 8 of the m-tile belong to lanes 16m + g and 16m + 8 + g
+        const uint4* r0 = reinterpret_cast<const uint4*>(
+            kb + static_cast<int64_t>(__shfl_sync(0xffffffffu, row, 16 * m + g)) * kst);
+        const uint4* r1 = reinterpret_cast<const uint4*>(
+            kb + static_cast<int64_t>(__shfl_sync(0xffffffffu, row, 16 * m + 8 + g)) * kst);
+        const float i0 = __shfl_sync(0xffffffffu, ci.y, 16 * m + g);
+        const float i1 = __shfl_sync(0xffffffffu, ci.y, 16 * m + 8 + g);
+        uint4 x0[4], x1[4];
 #pragma unroll
-      for (int m = 0; m < 2; ++m)
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-          const int src = 16 * m + 8 * hh + g;
-          ra[m][hh] = kw32 + static_cast<int64_t>(__shfl_sync(0xffffffffu, row, src)) * kst32;
-          ir[m][hh] = __shfl_sync(0xffffffffu, ci.y, src);
+        for (int s = 0; s < 4; ++s) {
+          x0[s] = __ldg(r0 + 4 * s + tq);
+          x1[s] = __ldg(r1 + 4 * s + tq);
         }
-      for (int a0 = a_lo; a0 < t; a0 += 16) {
-        float d[2][2][4];
+        float c0 = -INFINITY, c1 = -INFINITY;
+#pragma unroll 1
+        for (int a0 = a_lo; a0 < t; a0 += 8) {
+          // column g is admission a0 + g (past t: one that stands, its dots unused)
+          const int an = a0 + g < t ? a0 + g : a0;
+          const uint4* src = an < kAdmStage ? admk + an * kAdmStride
+                                            : reinterpret_cast<const uint4*>(kb + static_cast<int64_t>(adm[an]) * kst);
+          float d[2][4];
 #pragma unroll
-        for (int m = 0; m < 2; ++m)
+          for (int e = 0; e < 4; ++e) d[0][e] = d[1][e] = 0.f;
 #pragma unroll
-          for (int n = 0; n < 2; ++n)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) d[m][n][e] = 0.f;
-        // column g of n-tile n is admission a0 + 8n + g (zero past t)
-        const uint32_t* rb[2];
-        bool bv[2];
-#pragma unroll
-        for (int n = 0; n < 2; ++n) {
-          const int an = a0 + 8 * n + g;
-          bv[n] = an < t;
-          rb[n] = !bv[n] ? kw32
-                         : (an < kAdmStage ? admw + an * (4 * kAdmStride)
-                                           : kw32 + static_cast<int64_t>(adm[an]) * kst32);
-        }
-#pragma unroll
-        for (int s8 = 0; s8 < kHeadDim / 16; ++s8) {
-          uint32_t af[2][4];
-#pragma unroll
-          for (int m = 0; m < 2; ++m) {
-            af[m][0] = __ldg(ra[m][0] + 8 * s8 + tq);
-            af[m][1] = __ldg(ra[m][1] + 8 * s8 + tq);
-            af[m][2] = __ldg(ra[m][0] + 8 * s8 + tq + 4);
-            af[m][3] = __ldg(ra[m][1] + 8 * s8 + tq + 4);
+          for (int s = 0; s < 4; ++s) {
+            const uint4 y = src[4 * s + tq];
+            mma_bf16(d[0], x0[s].x, x1[s].x, x0[s].y, x1[s].y, y.x, y.y);
+            mma_bf16(d[1], x0[s].z, x1[s].z, x0[s].w, x1[s].w, y.z, y.w);
           }
-#pragma unroll
-          for (int n = 0; n < 2; ++n) {
-            const uint32_t b0 = bv[n] ? rb[n][8 * s8 + tq] : 0u;
-            const uint32_t b1 = bv[n] ? rb[n][8 * s8 + tq + 4] : 0u;
-#pragma unroll
-            for (int m = 0; m < 2; ++m) {
-              mma_bf16(d[m][n], af[m][0], af[m][1], af[m][2], af[m][3], b0, b1);
-            }
-          }
-        }
-        // element 2hh + e of d[m][n] is (row g + 8hh of m-tile m, column 2tq + e)
-        float rmax[2][2];
-#pragma unroll
-        for (int m = 0; m < 2; ++m) rmax[m][0] = rmax[m][1] = -INFINITY;
-#pragma unroll
-        for (int n = 0; n < 2; ++n)
+          // elements e and 2 + e: rows g and g + 8, admission a0 + 2tq + e
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
-            const int a = a0 + 8 * n + 2 * tq + e;
+            const int a = a0 + 2 * tq + e;
             if (a < t) {
               const float ia = adm_inv[a];
-#pragma unroll
-              for (int m = 0; m < 2; ++m)
-#pragma unroll
-                for (int hh = 0; hh < 2; ++hh)
-                  rmax[m][hh] = fmaxf(rmax[m][hh], d[m][n][2 * hh + e] * ir[m][hh] * ia);
+              c0 = fmaxf(c0, (d[0][e] + d[1][e]) * i0 * ia);
+              c1 = fmaxf(c1, (d[0][2 + e] + d[1][2 + e]) * i1 * ia);
             }
           }
+        }
 #pragma unroll
-        for (int m = 0; m < 2; ++m)
-#pragma unroll
-          for (int hh = 0; hh < 2; ++hh) {
-            rmax[m][hh] = fmaxf(rmax[m][hh], __shfl_xor_sync(0xffffffffu, rmax[m][hh], 1));
-            rmax[m][hh] = fmaxf(rmax[m][hh], __shfl_xor_sync(0xffffffffu, rmax[m][hh], 2));
-          }
-        // lane 16m + 8hh + gg takes row (m, gg + 8hh) from lane 4gg
-        const int src = 4 * (lane & 7);
-        const float r00 = __shfl_sync(0xffffffffu, rmax[0][0], src);
-        const float r01 = __shfl_sync(0xffffffffu, rmax[0][1], src);
-        const float r10 = __shfl_sync(0xffffffffu, rmax[1][0], src);
-        const float r11 = __shfl_sync(0xffffffffu, rmax[1][1], src);
-        const float mine = (lane >> 4) ? ((lane >> 3) & 1 ? r11 : r10) : ((lane >> 3) & 1 ? r01 : r00);
-        cm = fmaxf(cm, mine);
+        for (int o = 1; o <= 2; o <<= 1) {
+          c0 = fmaxf(c0, __shfl_xor_sync(0xffffffffu, c0, o));
+          c1 = fmaxf(c1, __shfl_xor_sync(0xffffffffu, c1, o));
+        }
+        // lane 16m + 8hh + gg takes its row's from lane 4gg
+        const float y0 = __shfl_sync(0xffffffffu, c0, 4 * (lane & 7));
+        const float y1 = __shfl_sync(0xffffffffu, c1, 4 * (lane & 7));
+        if ((lane >> 4) == m) cm = fmaxf(cm, (lane >> 3) & 1 ? y1 : y0);
       }
-      if (stale) {
-        cinv[my_idx] = make_float2(cm, ci.y);
+      if (want) {
+        cinv[my_idx].x = cm;
         v[my_idx] = fmaf(lambda2, cm, st[my_idx]);
         applied[my_idx] = static_cast<uint16_t>(t);
-        rescan();
+        rescan(t);
       }
     }
-    __syncthreads();
   };
 
   int32_t* order = P.order ? P.order + u.unit * B : nullptr;
   float* margins = P.margins ? P.margins + u.unit * B : nullptr;
   int t = 0;
+  bool again = false, all = false, second = false;   // second: the search is for the runner-up
+  uint32_t best = 0;
+#pragma unroll 1
   while (t < nsel) {
-    block_best(my_key, my_idx, sh);
-    const int bi = static_cast<int>(sh.best_idx);
-    if (applied[bi] < t) {            // a stale bound: bring stale bests up to date, search again
-      refresh_stale_bests(t);
-      continue;
+    if (again) {
+      if (all)
+        refresh_all(t - 1);
+      else
+        refresh_bests(t);
     }
-    // bi is the full greedy's admission at step t
-    const float vstar = v[bi];
-    __syncthreads();                  // every thread has read v[bi] and applied[bi]
-    if (tid == 0) {
-      adm[t] = bi;
-      v[bi] = -INFINITY;
-      if (order) order[t] = bi;
-    }
-    if (t < kAdmStage && tid < kHeadDim / 8)
-      admk[t * kAdmStride + tid] =
-          __ldg(reinterpret_cast<const uint4*>(kb + static_cast<int64_t>(bi) * kst) + tid);
-    __syncthreads();
-    if (own == (bi % kAllThreads)) rescan();
-    if (margins) {
-      // the runner-up, brought up to date against admissions 0 .. t-1
-      for (;;) {
-        block_best(my_key, my_idx, sh);
-        const uint32_t si = sh.best_idx;
-        if (si == 0xFFFFFFFFu) {
-          if (tid == 0) margins[t] = INFINITY;
-          break;
-        }
-        if (applied[si] < t) {
-          refresh_stale_bests(t);
-          continue;
-        }
-        if (tid == 0) margins[t] = vstar - v[si];
-        break;
+    block_best(my_key, my_idx, my_cur, applied, t, sh);
+    again = sh.stale;                 // a bound: bring what could beat it up to date, search again
+    all = false;
+    if (again) continue;
+    if (!second) {
+      // the full greedy's admission at step t
+      const int bi = static_cast<int>(sh.best_idx);
+      best = sh.best_key;
+      if (own == (bi % kAllThreads)) {
+        v[bi] = -INFINITY;
+        rescan(t);
+        adm[t] = bi;
+        adm_inv[t] = cinv[bi].y;      // the admitted key's inverse norm
+        if (order) order[t] = bi;
       }
+      if (t < kAdmStage && tid < kHeadDim / 8)
+        admk[t * kAdmStride + tid] =
+            __ldg(reinterpret_cast<const uint4*>(kb + static_cast<int64_t>(bi) * kst) + tid);
+      second = margins != nullptr;
+      if (second) continue;           // against admissions 0 .. t-1 too
+    } else {
+      if (tid == 0)
+        margins[t] = sh.best_idx == 0xFFFFFFFFu ? INFINITY : unord_key_all(best) - unord_key_all(sh.best_key);
+      second = false;
     }
-    if (tid == 0) adm_inv[t] = cinv[bi].y;   // inverse norm of the admitted key
-    __syncthreads();
     ++t;
-    // lambda2 > 0: values grow with corr, so every candidate is brought up to date (by its owner)
-    if (!lazy && t < nsel) refresh_all(t - 1);
+    my_cur = 0;
+    // lambda2 > 0: values grow with corr, so every candidate is brought up to date
+    if (!lazy && t < nsel) {
+      again = all = true;
+      __syncthreads();                // the admitted key and its norm are in place
+    }
   }
 
   // 3. admitted positions ascending, then -1: entry a of the admission order goes to

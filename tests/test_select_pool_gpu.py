@@ -1,7 +1,7 @@
 """Pool sizes at the edges of the selector's greedy: one half of 128 slots and two, a slot short of a
 half and one past it, the largest pool whose dot products stand before the greedy (256) and the smallest
 beyond it; equal scores and repeated keys, whose ties go to the lower position; and the every-candidate
-selector's candidate counts around its warps' 32 rows and its block's 1024, with both signs of lambda2;
+selector's candidate counts around its warps' 32 rows and its block's 512, with both signs of lambda2;
 very small, very large and zero keys.
 Every admission is replayed through the oracle, margins included."""
 
