@@ -50,8 +50,8 @@ FALLBACK_HBM_GBS = 6800.0
 # from the ncu capture summarised in profiles/, valid only for the sources it was taken
 # on (sha256 over csrc/kve_score.cu and csrc/kve_host.cu, which sets the schedule); per
 # launch of the full workload.
-SCORE_TRAFFIC = {"source_sha256": "60b3a57416c0a61c7b7c3b1774a219755c992425eaef2ae96c39b9cac38a0974",
-                 "bytes_per_launch": 2172808960 + 74820352}
+SCORE_TRAFFIC = {"source_sha256": "055df5f11878ee7fa410ecb7b88eaa227d447f8e66c0c20854f1b953b5eb4cce",
+                 "bytes_per_launch": 2180140800 + 74893056}
 
 
 def _score_source_sha():

@@ -127,7 +127,8 @@ void fill_units(kve::Geometry* g, int64_t ctas) {
 // head where their window rows fill whole 32-row blocks of the score kernel in equal runs of
 // 8-row blocks (W = 8, 16 or 32), else 1 (a unit per query head). The window rows of a KV head's
 // query heads are the default plan's 128 rows at most, so one pass over K serves them all: 32
-// layers of 4096 tokens take 83 us of score kernel against 264 with a unit per query head.
+// layers of 4096 tokens take 101 us of score kernel against 248 with a unit per query head, 8192
+// tokens 171 against 482.
 int32_t score_heads(const kve::Geometry& g) {
   const int rows = g.group * g.window;
   return g.uheads == g.hq && g.group == 4 && g.window % 8 == 0 && (rows == 32 || rows == 64 || rows == 128) ? 4 : 1;
@@ -140,7 +141,7 @@ int32_t score_heads(const kve::Geometry& g) {
 // width) stay in L2 for the phase-1 re-read. Where a round's items are short (a unit length
 // whose splits divide the CTA count only with items of half the size), the merge would not have
 // landed by then, and one round more still streams no more than that: 32 layers of 20011 tokens
-// (items of 4 tiles, 20 MB a round) take 476 us of score kernel against 507.
+// (items of 4 tiles, 20 MB a round) take 400 us of score kernel against 505.
 int32_t score_lag(const kve::Geometry& g, int64_t ctas) {
   int64_t span = 0, tiles = 0;   // tiles: of the longest item
   const int64_t units_per_req = static_cast<int64_t>(g.num_layers) * g.uheads;

@@ -23,10 +23,10 @@
 // unit's items run side by side in one round (the host picks the items per unit so
 // that rounds hold whole units). A CTA runs the phase-0 pass of its round-j item,
 // then the phase-1 pass of its round-(j - lag) item. A unit's items span at most
-// lag - 1 rounds (the host computes lag from the geometry), so every phase-1 item
-// waits only on phase-0 work that comes earlier in every CTA's sequence: there is
-// no circular wait. Between the two passes over an item's K tiles the GPU streams
-// about one round of other tiles, far less than L2 holds, so the phase-1 pass
+// lag - 1 rounds (the host computes lag from the geometry; one more where rounds
+// are short), so every phase-1 item waits only on phase-0 work that comes earlier
+// in every CTA's sequence: there is no circular wait. Between the two passes over an item's K tiles the GPU streams
+// about one or two rounds of other tiles, less than L2 holds, so the phase-1 pass
 // reads its tiles from L2. Every cross-CTA wait is bounded and a timeout is
 // reported as KVE_ETIMEOUT.
 //
@@ -79,8 +79,9 @@ constexpr uint32_t kMNSbo = 1024;
 // the column pass also streams V and accumulates O^T on the tensor cores: a column
 // tile's K stage holds its probabilities P^T until the O^T MMA has read them, so the
 // shared memory goes to 3 K stages and 2 V stages with a single Q buffer and a merge
-// buffer for 16 partials (measured: 1.84 ms per call at L = 32768 against 1.97 ms with
-// 2 Q buffers, 2 K stages and 8 partials); 3 score accumulators and the O^T accumulator
+// buffer for 16 partials (1.84 ms per call at L = 32768 against 1.97 ms with 2 Q buffers, 2 K
+// stages and 8 partials, both before the output's partials were summed by attn_finish_kernel as
+// it stands, 1.28 ms now); 3 score accumulators and the O^T accumulator
 // in TMEM columns 384..511.
 // kRB: 32-row blocks that hold the unit's window rows, 1, 2 or 4. With one block the keys are the
 // M side of the MMA in both passes and N is 32; otherwise Q is loaded as 128 rows and the column
@@ -277,7 +278,7 @@ __device__ __forceinline__ float2 merge_halves(float2 a, float2 b, bool hi, int 
 // g + 8, g + 16, g + 24 of its warp's 32 and the rows 8c + 2t, 8c + 2t + 1; it keeps (m, Z) of
 // those 8 rows over its keys, and the warp merges them at the end of the item. Both passes of a
 // tile then cost a quarter of the exponentials, and a quarter of the MMA's N: 32 layers of 15611
-// tokens with 8 x 4 rows take 248 us of score kernel against 289.
+// tokens with 8 x 4 rows take 262 us of score kernel against 289.
 __device__ __forceinline__ bool rowstats_by_key(const ScoreParams& P, ScoreCtl& ctl,
                                                 const ItemDesc& d, uint32_t slot, uint32_t& ai) {
   constexpr int kAccBufs = Cfg<1, false>::kAccBufs;
