@@ -646,7 +646,7 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
     if (pass > 0)
       for (int b = tid; b < nb; b += NT) hist[b] = 0;
     __syncthreads();
-    const uint32_t prefix = sh.prefix;
+    const uint32_t prefix = sh.prefix, need = sh.need;   // (before the barriers: one thread replaces them)
     if (pass > 0 && staged) {
       for (uint32_t e = tid; e < ncand; e += NT) {
         const uint32_t k = cand_k[e];
@@ -675,7 +675,6 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
     if (b0 < nb)
       for (int b = 0; b < per; ++b) mine += hist[b0 + b];
     const uint32_t above = block_excl_suffix<NT>(mine, sh);
-    const uint32_t need = sh.need;
     if (b0 < nb && above < need && above + mine >= need) {
       uint32_t acc = above;
       for (int b = per - 1; b >= 0; --b) {
