@@ -85,6 +85,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64
   return mbar_try_wait(bar, parity) || mbar_wait_slow(bar, parity, limit_ns, abort);
 }
 
+// Bounded wait of a whole warp: the outcome is the same for every lane and the lanes are together
+// again behind it. Lanes may leave mbar_wait at different times (at the first poll, or from the
+// loop), and a .sync.aligned instruction behind it needs all of them.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns, volatile int* abort) {
+  const bool ok = mbar_wait(bar, parity, limit_ns, abort);
+  return __all_sync(0xffffffffu, ok);
+}
+
 // Two waits whose first polls are issued together, so that their latencies overlap when
 // both barriers are ready (the common case on a critical path); otherwise the bounded
 // waits above, one after the other.

@@ -173,14 +173,6 @@ __device__ __forceinline__ void set_error(const ScoreParams& P, ScoreCtl& ctl, u
   ctl.abort = 1;
 }
 
-// Bounded wait whose outcome is the same for every lane of the warp, so that a
-// warp never splits in front of a .sync.aligned instruction.
-__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, uint64_t limit,
-                                          volatile int* abort) {
-  const bool ok = mbar_wait(bar, parity, limit, abort);
-  return __all_sync(0xffffffffu, ok);
-}
-
 // Merge of two (m, Z) pairs in log2 units: Z counts 2^(x - m).
 __device__ __forceinline__ float2 merge_mz(float2 a, float2 b) {
   const float m = fmaxf(a.x, b.x);
@@ -357,6 +349,7 @@ __device__ __forceinline__ void col_half_values(const ScoreParams& P, const Scor
                                                 const float4* nb4, uint32_t taddr, int h0, int n,
                                                 int rel, float (&v)[64]) {
   const int nh = kFull ? 64 : (n - h0 < 64 ? n - h0 : 64);   // rows of this half, >= 1
+  __syncwarp();   // (the first half's causal mask is a branch per lane)
   tmem_ld32(taddr + h0, v);
   if (kFull || nh > 32) {
     tmem_ld32(taddr + h0 + 32, v + 32);
@@ -468,6 +461,7 @@ __device__ __forceinline__ float2 colstats_exact(const ScoreParams& P, const Sco
   for (int i = 0; i < rows; i += 32) {
     const int nh = rows - i < 32 ? rows - i : 32;
     float v[32];
+    __syncwarp();   // (the terms of the chunk before are formed behind branches per lane)
     tmem_ld32(taddr + static_cast<uint32_t>(r0 + i), v);
     tmem_wait_ld(v);
     float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
@@ -618,10 +612,8 @@ __device__ __forceinline__ bool colstats_by_fragment(const ScoreParams& P, Score
           float q = (hi ? Q[h][1] : Q[h][0]) + __shfl_xor_sync(0xffffffffu, hi ? Q[h][0] : Q[h][1], 2);
           a += __shfl_xor_sync(0xffffffffu, a, 1);
           q += __shfl_xor_sync(0xffffffffu, q, 1);
-          if ((tq & 1) == hh) {
-            S1[h] = a;
-            m2[h] = q;
-          }
+          S1[h] = (tq & 1) == hh ? a : S1[h];
+          m2[h] = (tq & 1) == hh ? q : m2[h];
         }
       }
       // The one-pass form loses about (sum A'^2) * 2^-19 to rounding. It is kept while

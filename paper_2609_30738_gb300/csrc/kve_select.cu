@@ -215,11 +215,12 @@ __device__ __forceinline__ bool gram_form(SelSmall<NT>& sh, uint8_t* keys, int n
     }
     tc_commit(bar);
   };
-  auto wait = [&](int i) { return mbar_wait(&sh.gram_bar[i], 0u, kGramWaitNs, &sh.abort); };
+  auto wait = [&](int i) { return warp_wait(&sh.gram_bar[i], 0u, kGramWaitNs, &sh.abort); };
   // after a wait that ran out: the products under way are waited for once more
   auto give_up = [&](int first, int last) {
-    if (threadIdx.x == 0)
-      for (int i = first; i <= last; ++i) wait(i);
+    if (threadIdx.x == 0) {
+      for (int i = first; i <= last; ++i) mbar_wait(&sh.gram_bar[i], 0u, kGramWaitNs, &sh.abort);
+    }
     __syncthreads();
     return false;
   };
@@ -338,6 +339,7 @@ __device__ __forceinline__ void gram_greedy(SelSmall<NT>& sh, const float* g01, 
       const uint32_t wsec = __reduce_max_sync(0xffffffffu, mine ? (second ? k[0] : k[1]) : key);
       if (lane == 0) sh.wsec[t & 1][warp] = wsec;
     }
+    __syncwarp();
     named_bar_sync(1, 128);
     const uint4 w01 = sh.win[t & 1][0], w23 = sh.win[t & 1][1];
     // the largest key, then the smallest tie key
@@ -353,6 +355,7 @@ __device__ __forceinline__ void gram_greedy(SelSmall<NT>& sh, const float* g01, 
     const float tm = tmem_ld1(tcol + static_cast<uint32_t>(js));
     const float of = js < 128 ? g01[jj * kGramPitch + i] : g01[i * kGramPitch + jj];
     const float2 inv_j = inv[js];
+    tmem_wait_ld();   // (before any branch per lane: aligned, like the load)
     if (i == 0) ties[t] = btie;
     if (want_second && i == 0) {
       // runner-up: the other warps' best and the winning warp's second
@@ -365,7 +368,6 @@ __device__ __forceinline__ void gram_greedy(SelSmall<NT>& sh, const float* g01, 
     }
     s[0].active = s[0].active && i != js;
     s[1].active = s[1].active && i + 128 != js;
-    tmem_wait_ld();
     const float d0 = js < 128 ? tm : of, d1 = js < 128 ? of : tm;
     s[0].corr = fmaxf(s[0].corr, cosine(d0, s[0].inv, inv_j));
     s[1].corr = fmaxf(s[1].corr, cosine(d1, s[1].inv, inv_j));
@@ -804,10 +806,10 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
   // same). Should that ever fail, the pool would hold unwritten slots: the unit is then
   // reported through the error word and gets no selection.
   if (n_above + needT != static_cast<uint32_t>(C) || needT > n_eq || needT == 0u) {
-    no_selection(kErrCheck);
     if constexpr (kGram) {
       if (warp == 0) tmem_dealloc(sh.tmem, kGramCols);
     }
+    no_selection(kErrCheck);
     return;
   }
   if (n_eq <= kTieCap) {

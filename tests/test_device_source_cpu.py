@@ -1,0 +1,60 @@
+"""Rules of the device code that a run does not show when they are broken (what follows is undefined
+rather than wrong each time), checked on the sources."""
+
+import glob
+import os
+import re
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2609_30738_gb300", "csrc")
+KERNELS = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
+
+
+def _code(path):
+    """The file's text with its comments and strings blanked out."""
+    text = open(path).read()
+    return re.sub(r'//[^\n]*|/\*.*?\*/|"(?:\\.|[^"\\\n])*"', lambda m: re.sub(r"[^\n]", " ", m.group()), text,
+                  flags=re.S)
+
+
+def _function(code, name):
+    """Text of the body of function `name`."""
+    at = re.search(r"\b%s\s*\([^;{]*\)\s*\{" % name, code).end()
+    depth, end = 1, at
+    while depth:
+        depth += {"{": 1, "}": -1}.get(code[end], 0)
+        end += 1
+    return code[at:end - 1]
+
+
+def _headers(code, at):
+    """What stands before each block that is open at position `at`, and the statement up to it."""
+    open_at, depth = [], 0
+    for i in range(at - 1, -1, -1):
+        if code[i] == "}":
+            depth += 1
+        elif code[i] == "{":
+            if depth:
+                depth -= 1
+            else:
+                open_at.append(i)
+    starts = [at] + open_at
+    return [re.split(r"[;{}]", code[:i])[-1] for i in starts]
+
+
+@pytest.mark.parametrize("path", KERNELS, ids=os.path.basename)
+def test_whole_warps_wait_together(path):
+    # the lanes of a warp may leave a bounded wait at different times: code that a whole warp runs
+    # waits by warp_wait, which brings them together again for the aligned instructions behind it
+    code = _code(path)
+    for m in re.finditer(r"\bmbar_wait2?\(", code):
+        one = r"(lane|threadIdx\.x|tid)\s*==\s*0"
+        assert any(re.search(one, h) for h in _headers(code, m.start())), code[:m.start()].count("\n") + 1
+
+
+def test_greedy_has_no_branch_between_tmem_load_and_wait():
+    body = _function(_code(os.path.join(CSRC, "kve_select.cu")), "gram_greedy")
+    between = re.search(r"tmem_ld1\((.*?)tmem_wait_ld\(", body, flags=re.S).group(1)
+    assert not re.search(r"\b(if|for|while)\b", between)
