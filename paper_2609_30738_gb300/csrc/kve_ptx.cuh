@@ -270,10 +270,10 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
 }
 
 // One fp32 column of this warp's 32 TMEM lanes.
-__device__ __forceinline__ float tmem_ld1(uint32_t taddr) {
+__device__ __forceinline__ void tmem_ld1(uint32_t taddr, float* v) {
   uint32_t r;
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr));
-  return __uint_as_float(r);
+  *v = __uint_as_float(r);
 }
 
 // Fragment loads of 16 TMEM lanes (taddr's lane and the 15 after it; the first or second
@@ -308,29 +308,14 @@ __device__ __forceinline__ void tmem_ld16_x8(uint32_t taddr, float* v) {
   for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
 }
 
-__device__ __forceinline__ void tmem_wait_ld() {
+// Wait for this warp's TMEM loads; `v` names the registers that they fill, so that nothing that
+// reads them can be scheduled before the wait (the empty statements stay behind it, and they are
+// where the values come from; they cost no instruction).
+template <int N>
+__device__ __forceinline__ void tmem_wait_ld(float (&v)[N]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// The same wait, naming the registers that the pending loads fill: nothing that reads them
-// can be scheduled before it.
-__device__ __forceinline__ void tmem_wait_ld(float (&v)[16]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]),
-                 "+f"(v[6]), "+f"(v[7]), "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]),
-                 "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15])
-               :: "memory");
-}
-
-__device__ __forceinline__ void tmem_wait_ld(float (&v)[32]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]),
-                 "+f"(v[6]), "+f"(v[7]), "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]),
-                 "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15]), "+f"(v[16]), "+f"(v[17]),
-                 "+f"(v[18]), "+f"(v[19]), "+f"(v[20]), "+f"(v[21]), "+f"(v[22]), "+f"(v[23]),
-                 "+f"(v[24]), "+f"(v[25]), "+f"(v[26]), "+f"(v[27]), "+f"(v[28]), "+f"(v[29]),
-                 "+f"(v[30]), "+f"(v[31])
-               :: "memory");
+#pragma unroll
+  for (int j = 0; j < N; ++j) asm volatile("" : "+f"(v[j]));
 }
 
 // ---------------------------------------------------------------- math

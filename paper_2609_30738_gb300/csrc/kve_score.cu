@@ -210,7 +210,7 @@ __device__ __forceinline__ bool rowstats_by_row(const ScoreParams& P, ScoreCtl& 
     const uint32_t taddr = ctl.tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + ab * 128u;
 #pragma unroll
     for (int c = 0; c < 4; ++c) tmem_ld32(taddr + 32u * c, v + 32 * c);
-    tmem_wait_ld();
+    tmem_wait_ld(v);
     tc_fence_before();
     __syncwarp();
     if (lane == 0) mbar_arrive(&ctl.acc_empty[ab]);
@@ -357,7 +357,7 @@ __device__ __forceinline__ void col_half_values(const ScoreParams& P, const Scor
 #pragma unroll
     for (int r = 32; r < 64; ++r) v[r] = 0.f;   // not loaded: rows past n
   }
-  tmem_wait_ld();
+  tmem_wait_ld(v);
   const float2 a2 = make_float2(P.alpha, P.alpha);
 #pragma unroll
   for (int r = 0; r < 64; r += 4) {

@@ -352,10 +352,11 @@ __device__ __forceinline__ void gram_greedy(SelSmall<NT>& sh, const float* g01, 
     const int js = static_cast<int>((packed ? (btie & 511u) : btie) & (kGramCols - 1u));
     const int jj = js & 127;
     // the dots with slot js: within its half in TMEM (column js), across in g01
-    const float tm = tmem_ld1(tcol + static_cast<uint32_t>(js));
+    float tm[1];
+    tmem_ld1(tcol + static_cast<uint32_t>(js), tm);
     const float of = js < 128 ? g01[jj * kGramPitch + i] : g01[i * kGramPitch + jj];
     const float2 inv_j = inv[js];
-    tmem_wait_ld();   // (before any branch per lane: aligned, like the load)
+    tmem_wait_ld(tm);   // (before any branch per lane: aligned, like the load)
     if (i == 0) ties[t] = btie;
     if (want_second && i == 0) {
       // runner-up: the other warps' best and the winning warp's second
@@ -368,7 +369,7 @@ __device__ __forceinline__ void gram_greedy(SelSmall<NT>& sh, const float* g01, 
     }
     s[0].active = s[0].active && i != js;
     s[1].active = s[1].active && i + 128 != js;
-    const float d0 = js < 128 ? tm : of, d1 = js < 128 ? of : tm;
+    const float d0 = js < 128 ? tm[0] : of, d1 = js < 128 ? of : tm[0];
     s[0].corr = fmaxf(s[0].corr, cosine(d0, s[0].inv, inv_j));
     s[1].corr = fmaxf(s[1].corr, cosine(d1, s[1].inv, inv_j));
   }

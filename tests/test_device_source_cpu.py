@@ -58,3 +58,12 @@ def test_greedy_has_no_branch_between_tmem_load_and_wait():
     body = _function(_code(os.path.join(CSRC, "kve_select.cu")), "gram_greedy")
     between = re.search(r"tmem_ld1\((.*?)tmem_wait_ld\(", body, flags=re.S).group(1)
     assert not re.search(r"\b(if|for|while)\b", between)
+
+
+@pytest.mark.parametrize("path", KERNELS, ids=os.path.basename)
+def test_tmem_waits_name_what_was_loaded(path):
+    # a wait that does not name the loaded registers does not keep their readers behind it
+    waited = re.findall(r"\btmem_wait_ld\(([^()]*)\)", _code(path))
+    loaded = re.findall(r"\btmem_ld\w+\(", _code(path))
+    assert bool(waited) == bool(loaded) and all(w.strip() for w in waited)
+    assert not re.search(r"tmem_wait_ld\(\s*\)", _code(os.path.join(CSRC, "kve_ptx.cuh")))
