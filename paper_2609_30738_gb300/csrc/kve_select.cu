@@ -861,6 +861,11 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
   }
   __syncthreads();
   const float smax = fmaxf(unord_key(sh.maxkey), P.norm_eps);
+  // the key of a position, or null outside the unit (only after a failed consistency check): the
+  // one place where a pool position becomes an address
+  const auto key_row = [&](int pos) {
+    return pos >= 0 && pos < Lc ? reinterpret_cast<const uint4*>(P.k + u.k_off + pos * P.g.k_st) : nullptr;
+  };
   // candidate keys row-major in shared memory; a half-warp copies one 256-byte row,
   // coalesced
   {
@@ -871,13 +876,10 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
       const int r = (q * (NT / 32) + warp) * 2 + (lane >> 4);
       xr[q] = make_uint4(0, 0, 0, 0);
       if (r < C) {
-        const int pos = ppos[r];
-        if (pos >= 0 && pos < Lc) {
-          const uint4* src = reinterpret_cast<const uint4*>(P.k + u.k_off + pos * P.g.k_st);
+        if (const uint4* src = key_row(ppos[r]))
           xr[q] = __ldg(src + (lane & 15));
-        } else if (P.err) {
+        else if (P.err)
           atomicOr(P.err, kErrCheck);   // never read outside the unit's keys
-        }
       }
     }
 #pragma unroll
@@ -930,8 +932,8 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
         inv2[tid] = inv_sqrt2(ss);
       else if (tid < C) {
         // sums that tensor cores may flush or cut off: from the key itself
-        const uint4* src = reinterpret_cast<const uint4*>(P.k + u.k_off + ppos[tid] * P.g.k_st);
-        inv2[tid] = make_float2(row_inv_norm([&](int c) { return __ldg(src + c); }), 0.f);
+        const uint4* src = key_row(ppos[tid]);
+        inv2[tid] = make_float2(src ? row_inv_norm([&](int c) { return __ldg(src + c); }) : 0.f, 0.f);
       }
     }
     __syncthreads();

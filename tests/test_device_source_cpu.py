@@ -67,3 +67,13 @@ def test_tmem_waits_name_what_was_loaded(path):
     loaded = re.findall(r"\btmem_ld\w+\(", _code(path))
     assert bool(waited) == bool(loaded) and all(w.strip() for w in waited)
     assert not re.search(r"tmem_wait_ld\(\s*\)", _code(os.path.join(CSRC, "kve_ptx.cuh")))
+
+
+def test_select_reads_keys_inside_the_unit():
+    # a pool position becomes a key's address in one place, which checks it, and whoever uses that
+    # address looks at the outcome
+    body = _function(_code(os.path.join(CSRC, "kve_select.cu")), "select_kernel")
+    assert body.count("P.k +") == 1
+    assert re.search(r"key_row = .*?pos >= 0 && pos < Lc \?[^;]*P\.k \+[^;]*: nullptr;", body, flags=re.S)
+    used = re.findall(r"[^;{}]*\bkey_row\(ppos[^;{}]*;[^;]*;", body)
+    assert len(used) == 2 and all("if (const uint4* src" in s or "src ?" in s for s in used)
