@@ -393,10 +393,13 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
                        : dyn_smem;
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
+  wait_previous_kernel();   // mu and sigma come from the score kernel launched before
   if constexpr (kGram) {
-    // Allocated and relinquished first thing: the SM starts no second block of the kernel before
-    // this block has given up its right to allocate (measured: half the blocks of a 256-unit
-    // launch began 44 us late when this stood before the greedy).
+    // TMEM is not taken before that wait: the previous kernel of the stream may be a caller's that
+    // allocates TMEM itself after it has let its dependents start. Allocated and relinquished
+    // right after it: the SM starts no second block of the kernel before this block has given up
+    // its right to allocate (measured: half the blocks of a 256-unit launch began 44 us late when
+    // this stood before the greedy).
     if (warp == 0) {
       tmem_alloc(&sh.tmem, kGramCols);
       tmem_relinquish();
@@ -410,7 +413,6 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
     __syncthreads();
     tc_fence_after();
   }
-  wait_previous_kernel();   // mu and sigma come from the score kernel launched before
 
   const UnitInfo u = unit_info(P.g, blockIdx.x);
   const int W = P.g.window;

@@ -77,3 +77,16 @@ def test_select_reads_keys_inside_the_unit():
     assert re.search(r"key_row = .*?pos >= 0 && pos < Lc \?[^;]*P\.k \+[^;]*: nullptr;", body, flags=re.S)
     used = re.findall(r"[^;{}]*\bkey_row\(ppos[^;{}]*;[^;]*;", body)
     assert len(used) == 2 and all("if (const uint4* src" in s or "src ?" in s for s in used)
+
+
+@pytest.mark.parametrize("path", KERNELS, ids=os.path.basename)
+def test_dependent_launches_take_no_tmem_early(path):
+    # a kernel that may start while its predecessor runs holds no TMEM before that has finished: the
+    # predecessor can be a caller's kernel that still has to allocate its own
+    code = _code(path)
+    for name in set(re.findall(r"\b(\w+_kernel)\s*\(const", code)):
+        body = _function(code, name)
+        if "wait_previous_kernel(" in body and "tmem_alloc(" in body:
+            assert body.index("wait_previous_kernel(") < body.index("tmem_alloc("), name
+    if os.path.basename(path) == "kve_select.cu":
+        assert "tmem_alloc(" in _function(code, "select_kernel")
