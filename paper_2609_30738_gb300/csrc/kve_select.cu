@@ -958,6 +958,14 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
     }
     tc_fence_before();
     __syncthreads();
+    if (warp == 0) {
+      tc_fence_after();
+      tmem_dealloc(sh.tmem, kGramCols);
+    }
+    if (!formed) {   // (there are no tie keys to decode)
+      no_selection(kErrWait);
+      return;
+    }
     for (int t = tid; t < nsel; t += NT) {
       const uint32_t tie = static_cast<uint32_t>(adm_slot[t]);
       const int js = static_cast<int>(packed ? (tie & 511u) : tie);
@@ -965,15 +973,6 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
       adm[t] = pos;
       adm_slot[t] = js;
       if (order) order[t] = pos;
-    }
-    __syncthreads();
-    if (warp == 0) {
-      tc_fence_after();
-      tmem_dealloc(sh.tmem, kGramCols);
-    }
-    if (!formed) {
-      no_selection(kErrWait);
-      return;
     }
   } else {
   __syncthreads();

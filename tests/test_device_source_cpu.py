@@ -90,3 +90,11 @@ def test_dependent_launches_take_no_tmem_early(path):
             assert body.index("wait_previous_kernel(") < body.index("tmem_alloc("), name
     if os.path.basename(path) == "kve_select.cu":
         assert "tmem_alloc(" in _function(code, "select_kernel")
+
+
+def test_select_decodes_only_what_the_greedy_wrote():
+    # after a wait that ran out no admission was written: the unit leaves before its tie keys, which
+    # index the pool, are decoded
+    body = _function(_code(os.path.join(CSRC, "kve_select.cu")), "select_kernel")
+    at = body.index("gram_greedy<NT>(")
+    assert at < body.index("if (!formed)", at) < body.index("adm_slot[t]", at)
