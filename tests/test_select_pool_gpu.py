@@ -26,8 +26,9 @@ def _lib():
     kv_evict.library()
 
 
-def _check(L, B, factor, lam2, seed, flat=False, scale=1.0):
-    """Selection on given mu and sigma (flat: few distinct values, runs of equal keys; scale: of the keys)."""
+def _check(L, B, factor, lam2, seed, flat=False, scale=1.0, dims=None):
+    """Selection on given mu and sigma (flat: few distinct values, runs of equal keys; scale: of the keys; dims:
+    the keys' first elements alone, at norm 1)."""
     from paper_2609_30738_gb300 import kv_evict as K
     W, nl, hkv = 8, 2, 2
     spec = scaled(WORKLOADS["mistral-1layer-L2048"], num_layers=nl, num_q_heads=4, num_kv_heads=hkv, window=W,
@@ -40,6 +41,10 @@ def _check(L, B, factor, lam2, seed, flat=False, scale=1.0):
         mu, sigma = np.round(mu * 2) / 2 + np.float32(0.25), np.round(sigma * 2) / 2
         batch["k"][:, :, 1::2] = batch["k"][:, :, 0:1]      # every other key is one and the same
     mu, sigma = mu.astype(np.float32), sigma.astype(np.float32)
+    if dims:
+        head = batch["k"][..., :dims].float()
+        batch["k"].zero_()
+        batch["k"][..., :dims] = head / head.norm(dim=-1, keepdim=True)
     if scale != 1.0:
         batch["k"] *= scale
         batch["k"][:, :, 5::7] = 0
@@ -83,3 +88,14 @@ def test_every_candidate_edges(Lc, lam2):
 def test_pool_key_scales(scale, B):
     """Squared norms below, around and above the range in which they are read from the dots; zero keys."""
     _check(700, B, 4, -0.5, seed=B, scale=scale)
+
+
+@pytest.mark.parametrize("B", [30, 60])
+@pytest.mark.parametrize("dims,scale", [(8, 2.0 ** -64.75), (None, 2.0 ** 60)])
+def test_pool_key_scales_at_the_ends(dims, scale, B):
+    """Norms whose inverses' product leaves the floats' range (every norm 2^-64.75), and norms near the
+    largest whose squares still sum. At the small end a product of two elements keeps multiples of 2^-149:
+    8 of them truncated move a dot by at most 2^-146, and rounded a squared norm by 2^-147, so that a cosine
+    moves by (2^-146 + 2^-147) / 2^-129.5 = 1.6e-5 and two values' difference (lambda2 = -0.5) by as much:
+    below the replay's 1e-4."""
+    _check(700, B, 4, -0.5, seed=B, scale=scale, dims=dims)
