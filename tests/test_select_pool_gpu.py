@@ -99,3 +99,32 @@ def test_pool_key_scales_at_the_ends(dims, scale, B):
     moves by (2^-146 + 2^-147) / 2^-129.5 = 1.6e-5 and two values' difference (lambda2 = -0.5) by as much:
     below the replay's 1e-4."""
     _check(700, B, 4, -0.5, seed=B, scale=scale, dims=dims)
+
+
+@pytest.mark.parametrize("lam2", [-0.5, 0.6])
+@pytest.mark.parametrize("Lc", [240, 500, 600, 2081])
+def test_masked_tokens_come_last(Lc, lam2):
+    """Tokens masked by mu = -inf, with fewer others than the budget: the others first, then the masked ones
+    from the lowest position up, in each of the three selectors."""
+    from paper_2609_30738_gb300 import kv_evict as K
+    W, B = 8, 24
+    spec = scaled(WORKLOADS["mistral-1layer-L2048"], num_layers=1, num_q_heads=4, num_kv_heads=1, window=W,
+                  budget=B, candidate_factor=0, pool_kernel=1, seq_lens=[Lc + W])
+    batch = synth.make_batch(spec, seed=Lc, with_values=False)
+    rng = np.random.default_rng(Lc)
+    kept = rng.choice(np.arange(3, Lc), size=10, replace=False)
+    mu = np.full(Lc + W, -np.inf, np.float32)
+    mu[kept] = rng.random(10).astype(np.float32) + 0.5
+    plan = K.Plan(spec, [Lc + W])
+    bufs = K.Buffers(plan)
+    bufs.mu.copy_(torch.from_numpy(mu))
+    bufs.sigma.fill_(0.25)
+    bufs.ws.zero_()
+    l1, l2 = np.full(1, 0.5, np.float32), np.full(1, lam2, np.float32)
+    for margins in (bufs.margins, None):
+        plan.select(bufs.mu, bufs.sigma, batch["k"].cuda(), l1, l2, bufs.indices, bufs.ws, bufs.order, margins)
+        assert plan.status(bufs.ws) == K.KVE_OK
+        order = bufs.order.cpu().numpy()[0]
+        assert set(order[:10]) == set(kept)
+        assert list(order[10:]) == [p for p in range(Lc) if p not in set(kept)][:B - 10]
+        assert np.array_equal(bufs.indices.cpu().numpy()[0], np.sort(order))
