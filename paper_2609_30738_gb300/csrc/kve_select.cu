@@ -285,18 +285,34 @@ __device__ __forceinline__ float2 inv_sqrt2(float x) {
   return make_float2(y, 0.5f * y * r);
 }
 
-// dot * a * b with a and b in two floats each, rounded once. Takes a.x * b.x in [2^-100, 2^100].
+// dot * a * b with a and b in two floats each, rounded once. Takes a.x * b.x in [2^-120, 2^120].
 __device__ __forceinline__ float cosine(float dot, float2 a, float2 b) {
   const float p = a.x * b.x;
   const float e = fmaf(a.x, b.x, -p) + fmaf(a.x, b.y, a.y * b.x);
   return fmaf(dot, p, dot * e);
 }
 
-// The same for any a and b: a product of inverse norms that leaves the floats' range (both keys' norms
-// below 2^-64, or both near the largest) is not formed; the dot is scaled by one after the other.
-__device__ __forceinline__ float cosine_any(float dot, float2 a, float2 b) {
-  const float p = a.x * b.x;
-  return p >= 0x1p-100f && p <= 0x1p100f ? cosine(dot, a, b) : dot * a.x * b.x;
+// For a pool with norms outside inv_sqrt2's range: the inverse norms of its C slots scaled by one power
+// of two, so that cosine's products of two of them stay in 2^-100 .. 2^102 (where the pool's norms lie
+// up to 2^100 apart; beyond that the smallest keys' products give way). Returns the factor by which the
+// cosines shrink; the caller scales lambda2 by its inverse, so that the greedy's loop knows nothing of
+// it: a branch in that loop, or a second copy of it, cost a search over 14 profiles 3 to 5 %. All
+// threads; the scaled norms are in place behind the caller's next barrier.
+__device__ __forceinline__ float scale_inverse_norms(float2* inv, int C) {
+  float lo = INFINITY, hi = 0.f;
+  for (int c = 0; c < C; ++c) {
+    const float x = inv[c].x;
+    if (x > 0.f && x < INFINITY) {
+      lo = fminf(lo, x);
+      hi = fmaxf(hi, x);
+    }
+  }
+  int k = 0;
+  if (hi > 0.f) k = min(max(0, ilogbf(hi) + 1 - 50), ilogbf(lo) + 50);
+  const float f = exp2f(static_cast<float>(-k));
+  __syncthreads();   // (all of them have been read)
+  if (threadIdx.x < C) inv[threadIdx.x] = make_float2(inv[threadIdx.x].x * f, inv[threadIdx.x].y * f);
+  return f * f;
 }
 
 // The greedy over a pool of up to 256 slots whose dot products stand (gram_form): warps 0 .. 3,
@@ -314,8 +330,7 @@ __device__ __forceinline__ float cosine_any(float dot, float2 a, float2 b) {
 // 1.50e-8 and 5.39e-8 with four chains of two MMAs and norms of two fp32 chains; with those norms
 // and the one chain it was 1.71e-8 and 6.37e-8.
 // st: normalised base score; inv: inverse norm (of inactive slots: `active` false); tie: position
-// << 9 | slot, or the slot. any_norm: some norm lies outside the range of inv_sqrt2. ties[t] receives
-// admission t's tie key.
+// << 9 | slot, or the slot. ties[t] receives admission t's tie key.
 struct GreedySlot {
   float st, corr;
   float2 inv;
@@ -324,8 +339,8 @@ struct GreedySlot {
 };
 template <int NT, class Margin>
 __device__ __forceinline__ void gram_greedy(SelSmall<NT>& sh, const float* g01, const float2* inv, GreedySlot (&s)[2],
-                                            float lambda2, int nsel, bool packed, bool any_norm,
-                                            uint32_t* ties, bool want_second, Margin margin) {
+                                            float lambda2, int nsel, bool packed, uint32_t* ties,
+                                            bool want_second, Margin margin) {
   const int i = threadIdx.x, warp = i >> 5, lane = i & 31;
   const uint32_t tcol = sh.tmem + (static_cast<uint32_t>(warp * 32) << 16);
   for (int t = 0; t < nsel; ++t) {
@@ -378,13 +393,8 @@ __device__ __forceinline__ void gram_greedy(SelSmall<NT>& sh, const float* g01, 
     s[0].active = s[0].active && i != js;
     s[1].active = s[1].active && i + 128 != js;
     const float d0 = js < 128 ? tm[0] : of, d1 = js < 128 ? of : tm[0];
-    if (__builtin_expect(any_norm, 0)) {
-      s[0].corr = fmaxf(s[0].corr, cosine_any(d0, s[0].inv, inv_j));
-      s[1].corr = fmaxf(s[1].corr, cosine_any(d1, s[1].inv, inv_j));
-    } else {
-      s[0].corr = fmaxf(s[0].corr, cosine(d0, s[0].inv, inv_j));
-      s[1].corr = fmaxf(s[1].corr, cosine(d1, s[1].inv, inv_j));
-    }
+    s[0].corr = fmaxf(s[0].corr, cosine(d0, s[0].inv, inv_j));
+    s[1].corr = fmaxf(s[1].corr, cosine(d1, s[1].inv, inv_j));
   }
 }
 
@@ -954,7 +964,10 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
         outside = y != 0.f;
       }
     }
-    const bool any_norm = __syncthreads_or(outside) != 0;
+    if (__syncthreads_or(outside) != 0) {
+      lambda2 *= 1.0f / scale_inverse_norms(inv2, C);   // (powers of two)
+      __syncthreads();
+    }
     if (formed && warp < 4) {
       GreedySlot s[2];
 #pragma unroll
@@ -966,7 +979,7 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
         s[e].corr = 0.f;
         s[e].tie = s[e].active ? tie_key(slot) : 0xFFFFFFFFu;
       }
-      gram_greedy<NT>(sh, reinterpret_cast<const float*>(big), inv2, s, lambda2, nsel, packed, any_norm,
+      gram_greedy<NT>(sh, reinterpret_cast<const float*>(big), inv2, s, lambda2, nsel, packed,
                       reinterpret_cast<uint32_t*>(adm_slot), margins != nullptr,
                       [&](int t, uint32_t best, uint32_t sec) {
                         margins[t] = sec ? unord_key(best) - unord_key(sec) : INFINITY;
