@@ -886,11 +886,6 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
   }
   __syncthreads();
   const float smax = fmaxf(unord_key(sh.maxkey), P.norm_eps);
-  // the key of a position, or null outside the unit (only after a failed consistency check): the
-  // one place where a pool position becomes an address
-  const auto key_row = [&](int pos) {
-    return pos >= 0 && pos < Lc ? reinterpret_cast<const uint4*>(P.k + u.k_off + pos * P.g.k_st) : nullptr;
-  };
   // candidate keys row-major in shared memory; a half-warp copies one 256-byte row,
   // coalesced
   {
@@ -901,10 +896,13 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
       const int r = (q * (NT / 32) + warp) * 2 + (lane >> 4);
       xr[q] = make_uint4(0, 0, 0, 0);
       if (r < C) {
-        if (const uint4* src = key_row(ppos[r]))
+        const int pos = ppos[r];
+        if (pos >= 0 && pos < Lc) {
+          const uint4* src = reinterpret_cast<const uint4*>(P.k + u.k_off + pos * P.g.k_st);
           xr[q] = __ldg(src + (lane & 15));
-        else if (P.err)
+        } else if (P.err) {
           atomicOr(P.err, kErrCheck);   // never read outside the unit's keys
+        }
       }
     }
 #pragma unroll
@@ -958,8 +956,12 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
         inv2[tid] = inv_sqrt2(ss);
       else if (tid < C) {
         // sums that tensor cores may flush or cut off: from the key itself
-        const uint4* src = key_row(ppos[tid]);
-        const float y = src ? row_inv_norm([&](int c) { return __ldg(src + c); }) : 0.f;
+        const int pos = ppos[tid];
+        float y = 0.f;
+        if (pos >= 0 && pos < Lc) {   // (a slot that failed this above has a zero row: it comes here)
+          const uint4* src = reinterpret_cast<const uint4*>(P.k + u.k_off + pos * P.g.k_st);
+          y = row_inv_norm([&](int c) { return __ldg(src + c); });
+        }
         inv2[tid] = make_float2(y, 0.f);
         outside = y != 0.f;
       }
