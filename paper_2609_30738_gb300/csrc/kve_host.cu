@@ -85,20 +85,70 @@ int device_sms() {
 // Score items per unit for a unit of T tiles. Items hold at most kSplitTiles tiles.
 // The score kernel deals items to its CTAs round-robin, one round = one item per CTA,
 // so a split count that divides the CTA count (or is a multiple of it) makes every
-// round hold whole units; up to twice the minimum count is accepted for that. A call of fewer
-// than kSplitTiles tiles per CTA (total_tiles over all units) takes items of total_tiles / ctas
-// tiles, so that one round gives every CTA its share: one layer of 2048 tokens (8 units of 16
-// tiles) runs on 128 CTAs instead of 16.
-int32_t choose_splits(int64_t T, int64_t ctas, int64_t total_tiles) {
-  if (ctas > 0 && total_tiles < ctas * kSplitTiles) {
-    const int64_t per_item = (total_tiles + ctas - 1) / ctas;
-    return static_cast<int32_t>((T + per_item - 1) / per_item);
-  }
+// round hold whole units; up to twice the minimum count is accepted for that.
+int32_t choose_splits(int64_t T, int64_t ctas) {
   const int64_t kmin = (T + kSplitTiles - 1) / kSplitTiles;
   const int64_t kmax = std::min<int64_t>(T, 2 * kmin);
   for (int64_t k = kmin; ctas > 0 && k <= kmax; ++k)
     if (ctas % k == 0 || k % ctas == 0) return static_cast<int32_t>(k);
   return static_cast<int32_t>(kmin);
+}
+
+// What the busiest CTA does with the items of g's req_splits: its tiles and its items. Splits for
+// which tiles + items cannot stay below `limit` are not counted out: their tiles are a lower bound.
+struct CtaLoad {
+  int64_t tiles, items;
+};
+constexpr int kMaxCtas = 1024;
+
+CtaLoad busiest_cta(const kve::Geometry& g, int64_t ctas, int64_t total_tiles, int64_t limit) {
+  const int64_t units_per_req = static_cast<int64_t>(g.num_layers) * g.uheads;
+  int64_t items = 0, longest = 0, shortest = INT64_MAX;
+  for (int r = 0; r < g.n_req; ++r) {
+    const int64_t T = g.req_tiles[r], k = g.req_splits[r];
+    items += units_per_req * k;
+    longest = std::max<int64_t>(longest, (T + k - 1) / k);
+    shortest = std::min<int64_t>(shortest, T / k);
+  }
+  const int64_t rounds = (items + ctas - 1) / ctas;
+  if (rounds == 1) return {longest, 1};
+  if (ctas > kMaxCtas) return {longest * rounds, rounds};
+  const int64_t least = std::max(std::max(longest, rounds * shortest), (total_tiles + ctas - 1) / ctas);
+  if (least + rounds >= limit) return {least, rounds};
+  int32_t tiles[kMaxCtas] = {};
+  int64_t cta = 0;
+  for (int r = 0; r < g.n_req; ++r)
+    for (int64_t u = 0; u < units_per_req; ++u)
+      for (int32_t s = 0; s < g.req_splits[r]; ++s) {
+        int32_t t0, nt;
+        kve::item_range(g, {r, static_cast<uint32_t>(u), static_cast<uint32_t>(s)}, &t0, &nt);
+        tiles[cta] += nt;
+        cta = cta + 1 == ctas ? 0 : cta + 1;
+      }
+  return {*std::max_element(tiles, tiles + ctas), rounds};
+}
+
+// Splits of every request. A call of fewer than kSplitTiles tiles per CTA is a round or two of the
+// score kernel, and its time that of the busiest CTA: of the rule above and of items of 1 to
+// kSplitTiles tiles it takes what leaves that CTA the fewest tiles and items (an item costs about a
+// tile besides its tiles), never more tiles than the rule above. Score kernel, 8 KV heads, us with the
+// rule above / with items of total / CTAs tiles, whose count can pass the CTAs' / here: 1 layer of 2048
+// tokens 26.6 / 18.6 / 18.6, 2 of 9400 26.7 / 32.9 / 26.7, 4 of 3840 26.8 / 28.8 / 26.8, 6 of 2900
+// 30.5 / 27.7 / 27.6, 12 of 1500 32.5 / 32.2 / 26.7.
+void choose_all_splits(kve::Geometry* g, int64_t ctas, int64_t total_tiles) {
+  for (int r = 0; r < g->n_req; ++r) g->req_splits[r] = choose_splits(g->req_tiles[r], ctas);
+  if (ctas <= 0 || total_tiles >= ctas * kSplitTiles) return;
+  const CtaLoad rule = busiest_cta(*g, ctas, total_tiles, INT64_MAX);
+  CtaLoad best = rule;
+  kve::Geometry t = *g;
+  for (int32_t per_item = kSplitTiles; per_item >= 1; --per_item) {
+    for (int r = 0; r < g->n_req; ++r) t.req_splits[r] = (g->req_tiles[r] + per_item - 1) / per_item;
+    const CtaLoad c = busiest_cta(t, ctas, total_tiles, best.tiles + best.items);
+    if (c.tiles <= rule.tiles && c.tiles + c.items < best.tiles + best.items) {
+      best = c;
+      std::copy(t.req_splits, t.req_splits + g->n_req, g->req_splits);
+    }
+  }
 }
 
 // Unit and item tables of g for its requests (req_len), units per layer and CTAs.
@@ -110,8 +160,8 @@ void fill_units(kve::Geometry* g, int64_t ctas) {
     g->req_tiles[r] = static_cast<int32_t>((static_cast<int64_t>(g->req_len[r]) + kTileKeys - 1) / kTileKeys);
     total_tiles += units_per_req * g->req_tiles[r];
   }
+  choose_all_splits(g, ctas, total_tiles);
   for (int r = 0; r < g->n_req; ++r) {
-    g->req_splits[r] = choose_splits(g->req_tiles[r], ctas, total_tiles);
     g->req_unit_base[r] = units;
     g->req_item_base[r] = items;
     units += units_per_req;

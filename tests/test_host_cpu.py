@@ -298,3 +298,35 @@ def test_kv_strides_validation_without_gpu():
             p.set_kv_strides(None, bad)
         assert e.value.status == K.KVE_EINVAL
     assert K.library().kv_evict_plan_set_kv_strides(None, None, None) == K.KVE_EINVAL
+
+
+def _busiest_tiles(units, tiles, splits, ctas):
+    """Tiles of the busiest CTA: items dealt round-robin, a unit's runs rotated by its index."""
+    load = np.zeros(min(ctas, units * splits), np.int64)
+    item = 0
+    for u in range(units):
+        run = (np.arange(splits) + u) % splits
+        n = (run + 1) * tiles // splits - run * tiles // splits
+        np.add.at(load, (item + np.arange(splits)) % len(load), n)
+        item += splits
+    return int(load.max())
+
+
+@pytest.mark.parametrize("n_req", [1, 2])
+@pytest.mark.parametrize("layers", [1, 2, 3, 4, 5, 6, 8, 11, 16, 19, 32])
+def test_score_items_never_load_a_cta_more_than_the_plain_rule(layers, n_req):
+    """Calls of few tiles are cut into smaller items to reach every CTA: the busiest one never has more tiles
+    than with items of 8 tiles whose count per unit divides the CTA count (four layers of 3840 tokens once
+    took 160 items over 152 CTAs, 12 tiles on some instead of 8). The items of a plan are read off the size of
+    its window-output scratch, 64 KB an item."""
+    _need_lib()
+    from paper_2609_30738_gb300 import kv_evict as K
+    ctas = 152
+    for tiles in list(range(1, 40)) + [45, 52, 64, 74, 80, 100, 127, 128, 152, 190, 255, 256]:
+        plan = K.Plan(_spec(num_layers=layers), [128 * tiles - 3] * n_req)
+        units = 8 * layers * n_req
+        items = plan.score_attn_workspace() // 65536
+        assert items % units == 0
+        kmin = -(-tiles // 8)
+        plain = next((k for k in range(kmin, min(tiles, 2 * kmin) + 1) if ctas % k == 0 or k % ctas == 0), kmin)
+        assert _busiest_tiles(units, tiles, items // units, ctas) <= _busiest_tiles(units, tiles, plain, ctas), tiles
