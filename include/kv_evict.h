@@ -208,9 +208,11 @@ kve_status kv_evict_select(const kve_plan* plan, const float* mu,
 /* Steps 3 and 4 in one launch: exactly what kv_evict_select followed by
  * kv_evict_gather writes (indices, order, margins, k_out, v_out; the same arguments
  * and the same layouts), with the compact cache written by the selection's own CTA
- * for each unit: the kept key rows come from the copy the selection stages for its
- * cosines (Eq. 4), so only the values and the window rows are read again. v may be
- * page-locked host memory as for kv_evict_gather (and k as well). Returns KVE_EINVAL
+ * for each unit. Beside the values and the window rows it reads the kept key rows a
+ * second time where the candidate pool is 256 at most (they are in L2, just read for
+ * the cosines of Eq. 4; larger pools still hold them in shared memory). v may be
+ * page-locked host memory as for kv_evict_gather (and k as well: its pool's rows, its
+ * kept rows and its window rows then cross the host link). Returns KVE_EINVAL
  * on the conditions of either call. For a plan whose selection runs over every
  * candidate (candidate_factor 0 beyond 512 prefix tokens) the two steps stay two
  * launches. */

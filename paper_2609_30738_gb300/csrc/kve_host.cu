@@ -175,7 +175,9 @@ void fill_units(kve::Geometry* g, int64_t ctas) {
 
 // Query heads whose statistics one score unit of a per-query-head plan holds: the four of a KV
 // head where their window rows fill whole 32-row blocks of the score kernel in equal runs of
-// 8-row blocks (W = 8, 16 or 32), else 1 (a unit per query head). The window rows of a KV head's
+// 8-row blocks (W = 8, 16 or 32), else 1 (a unit per query head). Four is the group of every
+// configuration here and the one the kernel is built for; groups of another size would each need a
+// variant of their own and keep a unit per query head, as they had. The window rows of a KV head's
 // query heads are the default plan's 128 rows at most, so one pass over K serves them all: 32
 // layers of 4096 tokens take 101 us of score kernel against 248 with a unit per query head, 8192
 // tokens 171 against 482.
@@ -384,7 +386,8 @@ kve_status score_impl(const kve_plan* plan, const uint16_t* q_win, const uint16_
   if (sms <= 0) return KVE_ECUDA;
   CUtensorMap tm_q, tm_k, tm_v;
   const int64_t q_rows = static_cast<int64_t>(g.num_layers) * g.n_req * g.hq * g.window;
-  if (!encode_rows(&tm_q, q_win, q_rows, kve::score_q_rows(g.n_rows, v != nullptr)) || !encode_keys(&tm_k, k, g)) return KVE_ECUDA;
+  const int q_box = kve::score_q_rows(g.n_rows, v != nullptr);
+  if (!encode_rows(&tm_q, q_win, q_rows, q_box) || !encode_keys(&tm_k, k, g)) return KVE_ECUDA;
   if (v && !encode_keys(&tm_v, v, g, true)) return KVE_ECUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   uint8_t* w = static_cast<uint8_t*>(ws);

@@ -25,9 +25,9 @@
 // then the phase-1 pass of its round-(j - lag) item. A unit's items span at most
 // lag - 1 rounds (the host computes lag from the geometry; one more where rounds
 // are short), so every phase-1 item waits only on phase-0 work that comes earlier
-// in every CTA's sequence: there is no circular wait. Between the two passes over an item's K tiles the GPU streams
-// about one or two rounds of other tiles, less than L2 holds, so the phase-1 pass
-// reads its tiles from L2. Every cross-CTA wait is bounded and a timeout is
+// in every CTA's sequence: there is no circular wait. Between the two passes over an
+// item's K tiles the GPU streams about one or two rounds of other tiles, less than L2
+// holds, so the phase-1 pass reads its tiles from L2. Every cross-CTA wait is bounded and a timeout is
 // reported as KVE_ETIMEOUT.
 //
 // Roles: warp 0 walks the item sequence and issues TMA loads; warp 1 owns TMEM and
@@ -714,8 +714,7 @@ __device__ __forceinline__ bool colstats_with_output(const ScoreParams& P, Score
     // The one-pass form loses about (sum A'^2) * 2^-19 to rounding. It is kept while
     // sigma^2 >= kOnePassMin * mu^2, where that loss stays below 2e-4 of sigma^2;
     // otherwise (columns of nearly equal A, e.g. uniform attention) the warp takes
-    // the two-pass form over the same TMEM columns, halves combined by the pairwise
-    // update of the mean and the sum of squared deviations (Chan, Golub, LeVeque).
+    // the two-pass form over the same TMEM columns (colstats_exact).
     const bool exact = !(m2 * fn * fn >= kOnePassMin * (fn - 1.f) * S1 * S1);   // NaN-safe
     if (__any_sync(0xffffffffu, exact)) {
       const float m2x = colstats_exact(P, ctl, nb4, taddr, 0, n, rel).y;

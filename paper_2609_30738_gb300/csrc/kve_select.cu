@@ -8,7 +8,7 @@
 //     the top 4B tokens) by an MSB-first radix select with 12/12/8-bit digits;
 //     ties at the cut go to the lower positions;
 //  3. normalise s~ = s / max(max s, eps) (Eq. 5) and stage the candidate keys
-//     (bf16) and their inverse norms in shared memory;
+//     (bf16) in shared memory;
 //  4. admit min(B, C) candidates greedily (Eq. 5): value s~ + lambda2 corr, ties to
 //     the lower position (the argmax compares position << 9 | slot after the value);
 //     after every admission j, corr_i <- max(corr_i, cos(k_i, k_j)), which is Eq. 4
@@ -143,7 +143,8 @@ __device__ __forceinline__ uint32_t block_excl_suffix(uint32_t x, SelSmall<NT>& 
 
 // Step 4 in the selection's CTA (P.k_out set): unit u's compact cache [B + W][d] as the
 // gather kernel writes it. Rows r < nvalid are the kept candidates in ascending position
-// (rpos[r]; krow != null: their key rows are still staged in shared memory, row rslot[r]); rows
+// (rpos[r]; krow != null: their key rows are still staged in shared memory, row rslot[r], otherwise
+// they are read again); rows
 // m .. m+W-1 are the window tokens Lc .. L-1; every other row is zero. A half-warp
 // copies a 256-byte row with 16-byte accesses; all loads of a batch are in flight before
 // its first store. The copy is bit-exact.
@@ -325,10 +326,12 @@ __device__ __forceinline__ float scale_inverse_norms(float2* inv, int C) {
 // 82 at 32768.
 // The products are summed along one chain of eight MMAs, which truncates. The norms come from the
 // diagonal, the same chain, so that this bias cancels in the cosine, and the inverse norms are
-// kept in two floats, so that the cosine is rounded once. Error of the margins against 64 bits
-// (same mu and sigma, 3000 tokens): 1.20e-8 rms at lambda2 = -0.5 and 4.53e-8 at 0.6, against
-// 1.50e-8 and 5.39e-8 with four chains of two MMAs and norms of two fp32 chains; with those norms
-// and the one chain it was 1.71e-8 and 6.37e-8.
+// kept in two floats, so that the cosine is rounded once. Error of a difference of two correlations
+// against 64 bits (rms of 65000 admissions at lambda2 = -1 and 1, base scores all 0), beside that of
+// the form that larger pools take (four chains of two MMAs, norms of two fp32 chains): clustered keys
+// 2.3e-8 and 6.9e-8 (3.0e-8, 8.3e-8), independent Gaussian keys 1.19e-8 and 2.20e-8 (1.30e-8,
+// 2.56e-8), positive keys 6.0e-8 and 6.4e-8 (7.0e-8, 7.7e-8), keys that four elements dominate 5.7e-8
+// and 11.2e-8 (6.1e-8, 10.8e-8).
 // st: normalised base score; inv: inverse norm (of inactive slots: `active` false); tie: position
 // << 9 | slot, or the slot. ties[t] receives admission t's tie key.
 struct GreedySlot {
@@ -941,7 +944,8 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) select_kernel(const __g
     return ss > 0.f ? inv_sqrt(ss) : 0.f;
   };
   const auto tie_key = [&](int slot) {
-    return packed ? (static_cast<uint32_t>(ppos[slot]) << 9) | static_cast<uint32_t>(slot) : static_cast<uint32_t>(slot);
+    const uint32_t low = static_cast<uint32_t>(slot);
+    return packed ? (static_cast<uint32_t>(ppos[slot]) << 9) | low : low;
   };
   if constexpr (kGram) {
     // 5. greedy admissions on the pool's dot products
