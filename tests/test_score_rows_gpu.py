@@ -75,3 +75,9 @@ def test_equal_rows_take_the_exact_form(W, per_query_head):
     # (the mu-proportional floor of tests/parity.py's derivation: 1e-4 mu)
     base = scaled(WORKLOADS["mistral-1layer-L2048"], window=W, budget=8, num_q_heads=8, num_kv_heads=2)
     _check(scaled(base, num_layers=1, seq_lens=[300, 1500]), per_query_head, 43, zero_q=True, sigma_mu_floor=1e-4)
+
+
+@pytest.mark.parametrize("layers,L", [(12, 1500), (2, 9400), (3, 5000)])
+def test_calls_of_few_tiles(layers, L):
+    # items cut by the busiest CTA's load, on 152 CTAs: 288 and 304 items (two rounds), 144 (one)
+    _check(scaled(WORKLOADS["mistral-1layer-L2048"], num_layers=layers, seq_lens=[L], budget=8), False, 44)
