@@ -50,8 +50,8 @@ FALLBACK_HBM_GBS = 6800.0
 # from the ncu capture summarised in profiles/, valid only for the sources it was taken
 # on (sha256 over csrc/kve_score.cu and csrc/kve_host.cu, which sets the schedule); per
 # launch of the full workload.
-SCORE_TRAFFIC = {"source_sha256": "055df5f11878ee7fa410ecb7b88eaa227d447f8e66c0c20854f1b953b5eb4cce",
-                 "bytes_per_launch": 2180140800 + 74893056}
+SCORE_TRAFFIC = {"source_sha256": "bbdce8f442b0e4752edc22386cfede790ded94c46f9f5aa489510241c458687b",
+                 "bytes_per_launch": 2179785472 + 74721792}
 
 
 def _score_source_sha():
